@@ -513,6 +513,7 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     DevParams &P = h->P;
     P.n = n;
     P.nb = n / 4;
+    while ((4 << P.lnb) < n) ++P.lnb;      // n is a power of two
     P.nbe = (uint32_t)(P.nb * P.nb * P.nb);
     P.n_envs = n_envs;
     P.bound = cfg->bound;
@@ -538,13 +539,16 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
 
     mpm_status st;
     const int nbuf = cfg->pipeline == MPM_PIPELINE_FUSED ? 2 : 1;
-    for (int b = 0; b < nbuf; ++b) {
-        if ((st = dalloc_t(h, &h->fb.P[b].xi, N)) != MPM_OK) return bail(st);
-        if ((st = dalloc_t(h, &h->fb.P[b].f0, N)) != MPM_OK) return bail(st);
-        if ((st = dalloc_t(h, &h->fb.P[b].f1, N)) != MPM_OK) return bail(st);
-        if ((st = dalloc_t(h, &h->fb.P[b].f2, N)) != MPM_OK) return bail(st);
-    }
-    if (nbuf == 1) h->fb.P[1] = h->fb.P[0];
+    // both buffers of an array in one allocation (the second starts on a 256-byte boundary)
+    const size_t ps = (N + 63) & ~size_t(63);
+    h->fb.pstride = nbuf == 2 ? (uint32_t)ps : 0u;
+    h->fb.cstride = h->chunk_cap;
+    PState &P0 = h->fb.P[0], &P1 = h->fb.P[1];
+    if ((st = dalloc_t(h, &P0.xi, ps * nbuf)) != MPM_OK) return bail(st);
+    if ((st = dalloc_t(h, &P0.f0, ps * nbuf)) != MPM_OK) return bail(st);
+    if ((st = dalloc_t(h, &P0.f1, ps * nbuf)) != MPM_OK) return bail(st);
+    if ((st = dalloc_t(h, &P0.f2, ps * nbuf)) != MPM_OK) return bail(st);
+    P1 = {P0.xi + h->fb.pstride, P0.f0 + h->fb.pstride, P0.f1 + h->fb.pstride, P0.f2 + h->fb.pstride};
     if ((st = dalloc_t(h, &h->fb.vc.vc0, N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->fb.vc.vc1, N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->fb.vc.vc2, N)) != MPM_OK) return bail(st);
@@ -560,12 +564,15 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     P.envp = h->d_envp;
     P.env_off = h->d_env_off;
     if (cfg->pipeline == MPM_PIPELINE_FUSED) {
-        for (int b = 0; b < 2; ++b) {
-            if ((st = dalloc_t(h, &h->fb.chunks[b], h->chunk_cap)) != MPM_OK) return bail(st);
-            if ((st = dalloc_t(h, &h->fb.tabs[b], h->nblocks)) != MPM_OK) return bail(st);
-            if ((st = dalloc_t(h, &h->fb.alist[b], h->nblocks)) != MPM_OK) return bail(st);
-            if ((st = dalloc_t(h, &h->fb.inbox[b], (size_t)h->nblocks * kInbox)) != MPM_OK) return bail(st);
-        }
+        const size_t nblk = h->nblocks;
+        if ((st = dalloc_t(h, &h->fb.chunks[0], 2 * (size_t)h->chunk_cap)) != MPM_OK) return bail(st);
+        if ((st = dalloc_t(h, &h->fb.tabs[0], 2 * nblk)) != MPM_OK) return bail(st);
+        if ((st = dalloc_t(h, &h->fb.alist[0], 2 * nblk)) != MPM_OK) return bail(st);
+        if ((st = dalloc_t(h, &h->fb.inbox[0], 2 * nblk * kInbox)) != MPM_OK) return bail(st);
+        h->fb.chunks[1] = h->fb.chunks[0] + h->chunk_cap;
+        h->fb.tabs[1] = h->fb.tabs[0] + nblk;
+        h->fb.alist[1] = h->fb.alist[0] + nblk;
+        h->fb.inbox[1] = h->fb.inbox[0] + nblk * kInbox;
         for (int b = 0; b < 3; ++b)
             if ((st = dalloc_t(h, &h->fb.clist[b], h->nblocks)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.astamp, h->nblocks)) != MPM_OK) return bail(st);

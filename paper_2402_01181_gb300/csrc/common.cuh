@@ -32,7 +32,8 @@ struct EnvParams {
 // whole handle is block g % nbe of environment g / nbe.
 struct DevParams {
     int n;            // nodes per axis
-    int nb;           // 4x4x4 blocks per axis (n / 4)
+    int nb;           // 4x4x4 blocks per axis (n / 4, a power of two)
+    int lnb;          // log2 nb
     uint32_t nbe;     // blocks per environment (nb^3)
     int n_envs;
     int bound;        // sticky wall band
@@ -144,6 +145,13 @@ inline void launch_dependent(void (*kernel)(K...), dim3 grid, dim3 block, size_t
     cudaLaunchKernelEx(&cfg, kernel, args...);   // a failure is left for cudaGetLastError
 }
 
+// block coordinates inside its environment of global block b, by shifts
+__host__ __device__ __forceinline__ void block_coords(uint32_t b, int lnb, int &bx, int &by, int &bz) {
+    const uint32_t m = (1u << lnb) - 1u;
+    bx = (int)(b & m);
+    by = (int)((b >> lnb) & m);
+    bz = (int)((b >> (2 * lnb)) & m);
+}
 __host__ __device__ __forceinline__ uint32_t block_id(int bx, int by, int bz, int nb) {
     return (uint32_t)(bx + nb * (by + nb * bz));
 }

@@ -86,8 +86,8 @@ struct FusedSmem {
     uint32_t lane_first[27], lane_off[27];
     // per pass parity: per direction, each warp's count of it (one byte per
     // warp, so that a lane sums all warps' counts of its direction in one load)
-    static constexpr int NWP = NW <= 4 ? 4 : 8;
-    alignas(8) uint8_t wcnt[2][28][NWP];
+    static constexpr int NWP = NW <= 4 ? 4 : NW;
+    alignas(16) uint8_t wcnt[2][28][NWP];
     uint32_t ncand, total, out_base, chunk_first, npass, mask, bmax, wide;
 };
 
@@ -153,24 +153,26 @@ __device__ __forceinline__ uint32_t source_slot(const Smem &s, uint32_t ncand, u
 
 // Start copying the particle with logical index j into this thread's slot.
 template <class Smem>
-__device__ __forceinline__ void prefetch_particle(Smem &s, const PState &in, uint32_t ncand, uint32_t j, int tid,
-                                                  int set) {
-    const uint32_t src = source_slot(s, ncand, j);
-    cp_async16_cg(&s.pxi[set][tid], &in.xi[src]);
-    cp_async16_cg(&s.pf0[set][tid], &in.f0[src]);
-    cp_async16_cg(&s.pf1[set][tid], &in.f1[src]);
-    cp_async4(&s.pf2[set][tid], &in.f2[src]);
+__device__ __forceinline__ void prefetch_particle(Smem &s, const PState &base, uint32_t in_off, uint32_t ncand,
+                                                  uint32_t j, int tid, int set) {
+    const uint32_t src = in_off + source_slot(s, ncand, j);
+    cp_async16_cg(&s.pxi[set][tid], &base.xi[src]);
+    cp_async16_cg(&s.pf0[set][tid], &base.f0[src]);
+    cp_async16_cg(&s.pf1[set][tid], &base.f1[src]);
+    cp_async4(&s.pf2[set][tid], &base.f2[src]);
 }
 
 // Start copying global block b's grid region of G_k, its inbox, and its
 // environment's material and tool frames into buffer buf.
 template <int T, class Smem>
-__device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, const uint4 *__restrict__ inbox_in,
+__device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, const uint4 *__restrict__ inbox,
+                                               uint32_t blk_in,
                                                const float4 *__restrict__ Gcur, const DevParams &P,
                                                const ToolFrame *__restrict__ tools, int tid) {
-    const uint32_t e = b / P.nbe, bl = b % P.nbe;
     const int nb = P.nb, n = P.n;
-    const int bx = bl % nb, by = (bl / nb) % nb, bz = bl / (nb * nb);
+    const uint32_t e = b >> (3 * P.lnb);
+    int bx, by, bz;
+    block_coords(b, P.lnb, bx, by, bz);
     constexpr int kTw = (int)(sizeof(ToolFrame) / 16);   // 16-byte words per frame
     const int ntw = P.tstride * kTw;
     for (int q = tid; q < 216 + kInbox + 2 + ntw; q += T) {
@@ -181,7 +183,7 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
                        ok);
         } else if (q < 216 + kInbox) {
             const int x = q - 216;
-            cp_async16(&s.inbox[buf][x], &inbox_in[(size_t)b * kInbox + x], true);
+            cp_async16(&s.inbox[buf][x], &inbox[(size_t)(blk_in + b) * kInbox + x], true);
         } else if (q < 216 + kInbox + 2) {
             const int x = q - 216 - kInbox;
             cp_async16(reinterpret_cast<uint4 *>(&s.ep[buf]) + x, reinterpret_cast<const uint4 *>(&P.envp[e]) + x, true);
@@ -215,26 +217,21 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     const uint32_t step = *(volatile uint32_t *)&ctrl->step;
     const int par = step & 1, m3 = step % 3;
     const int m3n = (m3 + 1) % 3, m3c = (m3 + 2) % 3;
-    const PState in = par ? B.P[1] : B.P[0];
-    const PState out = par ? B.P[0] : B.P[1];
-    const Chunk *__restrict__ cin = par ? B.chunks[1] : B.chunks[0];
-    Chunk *__restrict__ cout = par ? B.chunks[0] : B.chunks[1];
-    const BlockTab *__restrict__ tin = par ? B.tabs[1] : B.tabs[0];
-    BlockTab *__restrict__ tout = par ? B.tabs[0] : B.tabs[1];
+    // the two buffers of each array lie in one allocation: the sub-step's parity
+    // is an index offset, the bases stay kernel parameters
+    const uint32_t in_off = par ? B.pstride : 0u, out_off = B.pstride - in_off;            // particle slots
+    const uint32_t chunk_in = par ? B.cstride : 0u, chunk_out = B.cstride - chunk_in;      // chunks
+    const uint32_t blk_in = par ? B.nblocks : 0u, blk_out = B.nblocks - blk_in;            // per-block tables
     const float4 *__restrict__ Gcur = B.G[m3];
     float4 *Gnext = B.G[m3n];
     float4 *Gclr = B.G[m3c];
-    const uint4 *__restrict__ inbox_in = par ? B.inbox[1] : B.inbox[0];
-    uint4 *__restrict__ inbox_out = par ? B.inbox[0] : B.inbox[1];
-    const uint32_t *__restrict__ act = B.alist[par];
-    uint32_t *act_next = B.alist[par ^ 1];
     // the active blocks: heavy ones listed from the front, light ones from the
     // back, and handed out heavy first so that the launch ends on short items
     const unsigned long long nhl = *(volatile unsigned long long *)&ctrl->nactive[par][0];
     const uint32_t nheavy = (uint32_t)nhl, nact = (uint32_t)nhl + (uint32_t)(nhl >> 32);
     const uint32_t acap = B.nblocks;
     auto item_block = [&](uint32_t it) -> uint32_t {
-        return it >= nact ? 0u : (it < nheavy ? act[it] : act[acap - 1u - (it - nheavy)]);
+        return it >= nact ? 0u : B.alist[0][blk_in + (it < nheavy ? it : acap - 1u - (it - nheavy))];
     };
     const uint32_t nclr = *(volatile uint32_t *)&ctrl->nclear[m3c];
     const uint32_t *__restrict__ clr = B.clist[m3c];
@@ -252,7 +249,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
         s.bids[0] = item_block(it);
     }
     __syncthreads();
-    if (s.items[0] < nact) prefetch_block<T>(s, 0, s.bids[0], inbox_in, Gcur, P, tools, tid);
+    if (s.items[0] < nact) prefetch_block<T>(s, 0, s.bids[0], B.inbox[0], blk_in, Gcur, P, tools, tid);
     // the P2G arena starts at zero; every flush returns the nodes it read to zero
     for (int q = tid; q < 4 * kArena; q += T) (&s.acc[0][0])[q] = 0;
     // 0. while the first block's inputs land: clear the grid blocks G_{k-1} touched,
@@ -267,9 +264,10 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
         if (item >= nact) break;
         const uint32_t b = s.bids[cb];                 // global block
         if (RECORD && tid == 0) rec.act[item] = b;
-        const uint32_t env = b / nbe, bl = b % nbe;     // environment, block inside it
-        const uint32_t eb0 = env * nbe;                 // first global block of the environment
-        const int bx = bl % nb, by = (bl / nb) % nb, bz = bl / (nb * nb);
+        const uint32_t env = b >> (3 * P.lnb);          // environment
+        const uint32_t eb0 = env * nbe;                 // its first global block
+        int bx, by, bz;
+        block_coords(b, P.lnb, bx, by, bz);
         const EnvParams &ep = s.ep[cb];
         const float m = ep.mass;
         // the next work item: the atomic is issued here and its result is
@@ -305,26 +303,36 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
             const uint4 *ib = s.inbox[cb];
             uint32_t nc = 0, carry = 0;
             if (ib[kInbox - 1].x != step) {
-                for (int base = 0; base < 27 * kNpMax; base += 32) {
-                    const int idx = base + lane;
+                // lane l takes direction 26 - l, all its source passes: one scan
+                uint32_t start[kNpMax], cnt[kNpMax], sum = 0, pos = 0;
+#pragma unroll
+                for (int p = 0; p < kNpMax; ++p) {
                     uint4 e = make_uint4(0u, 0u, 0u, 0u);
-                    if (idx < 27 * kNpMax) e = ib[(26 - (idx / kNpMax)) * kNpMax + (idx % kNpMax)];
-                    const bool ok = idx < 27 * kNpMax && e.z == step && e.y > 0u;
+                    if (lane < 27) e = ib[(26 - lane) * kNpMax + p];
+                    const bool ok = e.z == step && e.y > 0u;     // step >= 1
                     const unsigned bal = __ballot_sync(0xffffffffu, ok);
-                    const uint32_t cnt = ok ? e.y : 0u;
-                    uint32_t incl = cnt;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += y;
-                    }
-                    if (ok) {
-                        const uint32_t pos = nc + __popc(bal & ((1u << lane) - 1u));
-                        s.cand_start[pos] = e.x;
-                        s.cand_pre[pos] = carry + incl - cnt;
-                    }
+                    start[p] = e.x;
+                    cnt[p] = ok ? e.y : 0u;
+                    sum += cnt[p];
+                    pos += __popc(bal & ((1u << lane) - 1u));
                     nc += __popc(bal);
-                    carry += __shfl_sync(0xffffffffu, incl, 31);
                 }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                carry = __shfl_sync(0xffffffffu, incl, 31);
+                uint32_t pre = incl - sum;
+#pragma unroll
+                for (int p = 0; p < kNpMax; ++p)
+                    if (cnt[p] > 0u) {
+                        s.cand_start[pos] = start[p];
+                        s.cand_pre[pos] = pre;
+                        ++pos;
+                        pre += cnt[p];
+                    }
             } else {
                 // a source wrote more passes than the inbox holds: walk its run tables
                 uint32_t np = 0, first = 0;
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     const int d = 26 - lane;
                     const int sx = bx - dir_dx(d), sy = by - dir_dy(d), sz = bz - dir_dz(d);
                     if (sx >= 0 && sy >= 0 && sz >= 0 && sx < nb && sy < nb && sz < nb) {
-                        const BlockTab t = tin[eb0 + block_id(sx, sy, sz, nb)];
+                        const BlockTab t = B.tabs[0][blk_in + eb0 + block_id(sx, sy, sz, nb)];
                         if (t.stamp == step) { np = t.npass; first = t.first; }
                     }
                 }
@@ -351,7 +359,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     if (c < ncand) {
                         int l = 0;
                         while (l < 26 && s.lane_off[l + 1] <= c) ++l;
-                        r = cin[s.lane_first[l] + (c - s.lane_off[l])].run[26 - l];
+                        r = B.chunks[0][chunk_in + s.lane_first[l] + (c - s.lane_off[l])].run[26 - l];
                     }
                     uint32_t incl2 = r.y;
                     for (int o = 1; o < 32; o <<= 1) {
@@ -394,20 +402,20 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 err |= kErrCapacity;
                 t.stamp = 0; t.first = 0; t.npass = 0;
             }
-            tout[b] = t;
+            B.tabs[0][blk_out + b] = t;
             if (RECORD) rec.blk[item] = make_uint2(fit ? alloc_ob : 0u, fit ? total : 0u);
             s.out_base = fit ? alloc_ob : nparticles;
             s.chunk_first = fit ? alloc_cf : nchunk_cap;
         }
         // this thread's particle of the first pass, then the next block's inputs;
         // both land while this block computes
-        if (npass > 0 && (uint32_t)tid < total) prefetch_particle(s, in, ncand, (uint32_t)tid, tid, 0);
+        if (npass > 0 && (uint32_t)tid < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)tid, tid, 0);
         cp_async_commit();
         if (PD == 2) {   // and the second pass's
-            if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle(s, in, ncand, (uint32_t)(T + tid), tid, 1);
+            if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)(T + tid), tid, 1);
             cp_async_commit();
         }
-        if (s.items[cb ^ 1] < nact) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], inbox_in, Gcur, P, tools, tid);
+        if (s.items[cb ^ 1] < nact) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
         else cp_async_commit();
         const int ox = 4 * bx - 1, oy = 4 * by - 1, oz = 4 * bz - 1;   // arena origin
 
@@ -416,6 +424,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
             const bool valid = j < total;
             const int slot = (pass % GP) * T + tid;    // staging slot within the group
             int d = 31;
+            uint32_t bound = 0u;      // this particle's share of the group bound (float bits)
             float nxp = 0.f, nyp = 0.f, nzp = 0.f, idf = 0.f, Fn[9], Cm[9], vx = 0.f, vy = 0.f, vz = 0.f;
             // this pass's particle is in the slot; the next block's inputs may still be landing
             // every thread commits, in order: pass 0's particle, [PD = 2: pass 1's
@@ -508,7 +517,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 nzp = xi.z + P.dt * vz;
                 // every value read from the slot has been consumed: refill it with the
                 // next pass's particle
-                if (pass + PD < npass && jn < total) prefetch_particle(s, in, ncand, jn, tid, ps);
+                if (pass + PD < npass && jn < total) prefetch_particle(s, B.P[0], in_off, ncand, jn, tid, ps);
                 if (!finite3(nxp, nyp, nzp)) {
                     err |= kErrNumeric;
                     nxp = xi.x; nyp = xi.y; nzp = xi.z;
@@ -548,7 +557,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     const float b1 = fabsf(qy) + 2.f * (fabsf(A[3]) + fabsf(A[4]) + fabsf(A[5]));
                     const float b2 = fabsf(qz) + 2.f * (fabsf(A[6]) + fabsf(A[7]) + fabsf(A[8]));
                     const float bp = fmaxf(fmaxf(b0, b1), b2);
-                    atomicMax(&s.bmax, isfinite(bp) ? __float_as_uint(bp) : 0u);
+                    bound = isfinite(bp) ? __float_as_uint(bp) : 0u;
                 } else {
                     // moved further than one cell: scatter straight into G_{k+1}
                     s.st_base[slot] = -1;
@@ -587,45 +596,60 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
             // --- stable rank by direction within the pass: per-warp counts, then
             // every warp derives the offsets it needs from the whole table (one
             // barrier per pass; warp 0 also publishes the pass's runs)
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
+            uint32_t my_pos = (uint32_t)tid;              // position in the pass's output
+            bool moved = valid && d != 13;                // to a neighbour block
             uint8_t(*wc)[Smem::NWP] = s.wcnt[pass & 1];
+            unsigned peers = __ballot_sync(0xffffffffu, valid);
+            if (__any_sync(0xffffffffu, moved)) peers = __match_any_sync(0xffffffffu, d);
+            const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
             if (valid && rank == 0) wc[d][warp] = (uint8_t)__popc(peers);
-            __syncthreads();
+            bound = __reduce_max_sync(0xffffffffu, bound);
+            if (lane == 0 && bound > 0u) atomicMax(&s.bmax, bound);
+            // no particle of the pass left the block (most passes: a particle moves a
+            // small part of a cell per sub-step): the order stays, one run
+            moved = __syncthreads_or(moved);
             const uint32_t out_base = s.out_base, chunk_first = s.chunk_first;
-            uint32_t run = 0, before = 0;                 // lane l: pass total and earlier warps' count of direction l
-            if (lane < 27) {
-                // byte sums by one multiply (four counts of at most 32: no carries)
-                auto bsum = [](uint32_t x) { return (x * 0x01010101u) >> 24; };
-                if (Smem::NWP == 8) {
-                    const uint2 c = *reinterpret_cast<const uint2 *>(&wc[lane][0]);
-                    const uint32_t mlo = warp >= 4 ? 0xffffffffu : (1u << (8 * warp)) - 1u;
-                    const uint32_t mhi = warp <= 4 ? 0u : (1u << (8 * (warp - 4))) - 1u;
-                    run = bsum(c.x) + bsum(c.y);
-                    before = bsum(c.x & mlo) + bsum(c.y & mhi);
-                } else {
-                    const uint32_t c = *reinterpret_cast<const uint32_t *>(&wc[lane][0]);
-                    run = bsum(c);
-                    before = bsum(c & ((1u << (8 * warp)) - 1u));
-                }
-            }
-            uint32_t incl = run;
+            const uint32_t pbase = out_base + pass * T;
+            const uint32_t npass_valid = min((uint32_t)T, total - pass * T);
+            // lane l: the pass's particles in direction l (run), and those in directions
+            // up to l (incl)
+            uint32_t run = lane == 13 ? npass_valid : 0u, incl = npass_valid;
+            if (moved) {
+                uint32_t before = 0;                          // earlier warps' count of direction l
+                run = 0;
+                if (lane < 27) {
+                    // byte sums by one multiply (four counts of at most 32: no carries)
+                    auto bsum = [](uint32_t x) { return (x * 0x01010101u) >> 24; };
+                    const uint32_t *cw = reinterpret_cast<const uint32_t *>(&wc[lane][0]);
+                    uint32_t c[Smem::NWP / 4];
+                    if (Smem::NWP == 16) *reinterpret_cast<uint4 *>(c) = *reinterpret_cast<const uint4 *>(cw);
+                    else if (Smem::NWP == 8) *reinterpret_cast<uint2 *>(c) = *reinterpret_cast<const uint2 *>(cw);
+                    else c[0] = cw[0];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
+                    for (int q = 0; q < Smem::NWP / 4; ++q) {
+                        const int w = warp - 4 * q;      // earlier warps among this word's four
+                        const uint32_t mk = w >= 4 ? 0xffffffffu : w <= 0 ? 0u : (1u << (8 * w)) - 1u;
+                        run += bsum(c[q]);
+                        before += bsum(c[q] & mk);
+                    }
+                }
+                incl = run;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                my_pos = __shfl_sync(0xffffffffu, incl - run + before, d & 31) + rank;
             }
-            const uint32_t my_off = __shfl_sync(0xffffffffu, incl - run + before, d & 31);
             // this warp's column of the other parity is next written by this warp, in
             // the next pass; every warp's reads of it ended before the barrier above
             if (lane < 28) s.wcnt[(pass + 1) & 1][lane][warp] = 0u;
             if (warp == 0 && chunk_first + pass < nchunk_cap) {
-                const uint32_t pbase = out_base + pass * T;
                 if (lane < 27) {
-                    cout[chunk_first + pass].run[lane] = make_uint2(pbase + incl - run, run);
+                    B.chunks[0][chunk_out + chunk_first + pass].run[lane] = make_uint2(pbase + incl - run, run);
                     const int tx = bx + dir_dx(lane), ty = by + dir_dy(lane), tz = bz + dir_dz(lane);
                     if (run > 0u && tx >= 0 && ty >= 0 && tz >= 0 && tx < nb && ty < nb && tz < nb) {
-                        uint4 *dst = inbox_out + (size_t)(eb0 + block_id(tx, ty, tz, nb)) * kInbox;
+                        uint4 *dst = B.inbox[0] + (size_t)(blk_out + eb0 + block_id(tx, ty, tz, nb)) * kInbox;
                         if (pass < (uint32_t)kNpMax)
                             dst[lane * kNpMax + pass] = make_uint4(pbase + incl - run, run, step + 1, 0u);
                         else
@@ -635,7 +659,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 const unsigned nz = __ballot_sync(0xffffffffu, lane < 27 && run > 0);
                 if (lane == 0) s.mask |= nz;
             }
-            const uint32_t pos = out_base + pass * T + my_off + rank;
+            const uint32_t pos = pbase + my_pos;
             if (RECORD && valid && pos < nparticles) {
                 rec.xi[pos] = xi;
                 rec.f0[pos] = a0;
@@ -645,10 +669,10 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 rec.src[pos] = source_slot(s, ncand, j);
             }
             if (valid && pos < nparticles) {
-                out.xi[pos] = make_float4(nxp, nyp, nzp, idf);
-                out.f0[pos] = make_float4(Fn[0], Fn[1], Fn[2], Fn[3]);
-                out.f1[pos] = make_float4(Fn[4], Fn[5], Fn[6], Fn[7]);
-                out.f2[pos] = Fn[8];
+                B.P[0].xi[out_off + pos] = make_float4(nxp, nyp, nzp, idf);
+                B.P[0].f0[out_off + pos] = make_float4(Fn[0], Fn[1], Fn[2], Fn[3]);
+                B.P[0].f1[out_off + pos] = make_float4(Fn[4], Fn[5], Fn[6], Fn[7]);
+                B.P[0].f2[out_off + pos] = Fn[8];
                 if (WRITE_VC) store_vc(B.vc, pos, vx, vy, vz, Cm);
             }
 
@@ -781,9 +805,9 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     // particles enter from outside, which are light.
                     if (atomicExch(&B.astamp[tb], step + 1) != step + 1) {
                         if (lane == 13 && total_b > (uint32_t)T)
-                            act_next[atomicAdd(&ctrl->nactive[par ^ 1][0], 1u)] = tb;
+                            B.alist[0][blk_out + atomicAdd(&ctrl->nactive[par ^ 1][0], 1u)] = tb;
                         else
-                            act_next[acap - 1u - atomicAdd(&ctrl->nactive[par ^ 1][1], 1u)] = tb;
+                            B.alist[0][blk_out + acap - 1u - atomicAdd(&ctrl->nactive[par ^ 1][1], 1u)] = tb;
                     }
                 }
                 if (warp == NW - 2) mark_clear(B, tb, step + 1, m3n);

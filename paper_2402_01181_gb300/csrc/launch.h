@@ -124,6 +124,9 @@ struct FusedBufs {
     uint32_t *gstamp;         // per block: last sub-step it was put on a clear list
     Ctrl *ctrl;
     uint32_t nblocks;
+    // the second buffer of P, chunks, tabs, alist and inbox follows the first in
+    // one allocation: pstride slots, cstride chunks, nblocks blocks further on
+    uint32_t pstride, cstride;
 };
 // What a recording fused sub-step writes for the reverse mode (all device
 // arrays): each block's input particles in block-contiguous order (n
