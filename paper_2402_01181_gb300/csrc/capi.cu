@@ -259,6 +259,7 @@ mpm_status status_of(uint32_t err) {
     if (err & kErrNumeric) return fail(MPM_ERR_NUMERIC, "device: non-finite state or det F <= 0");
     if (err & kErrDomain) return fail(MPM_ERR_DOMAIN, "device: a particle stencil left the grid (clamped)");
     if (err & kErrCfl) return fail(MPM_ERR_CFL, "device: a particle moved more than one block in a sub-step");
+    if (err & kErrStall) return fail(MPM_ERR_TIMEOUT, "device: the wait between two sub-steps ran out");
     if (err & kErrCapacity) return fail(MPM_ERR_CAPACITY, "device: run-table or particle-count capacity exceeded");
     return MPM_OK;
 }
@@ -398,24 +399,25 @@ mpm_status enqueue_error_copy(mpm_handle *h) {
 mpm_status issue_substeps(mpm_handle *h, int nsub, bool write_vc_last, cudaStream_t st) {
     const DevParams P = h->P;
     const uint32_t n = (uint32_t)h->n;
+    if (is_fused(h)) {
+        launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->fused_grid, h->kernel_config, st);
+        CK(cudaGetLastError());
+        return MPM_OK;
+    }
     for (int k = 0; k < nsub; ++k) {
         const ToolFrame *fr = h->d_frames + (size_t)k * h->n_envs * h->tstride;
-        const bool vc = write_vc_last && k == nsub - 1;
-        if (is_fused(h)) {
-            launch_fused_step(P, h->fb, fr, vc, h->fused_grid, h->kernel_config, st);
-        } else {
-            CK(cudaMemsetAsync(h->fb.G[0], 0, sizeof(float4) * (size_t)h->P.n * h->P.n * h->P.n, st));
-            launch_p2g_scatter(P, h->fb.P[0], h->fb.vc, n, h->fb.G[0], h->fb.ctrl, h->elem_grid, st);
-            launch_grid_update_dense(P, h->fb.G[0], fr, h->elem_grid, st);
-            launch_g2p_split(P, h->fb.P[0], h->fb.vc, n, h->fb.G[0], h->fb.ctrl, h->elem_grid, st);
-        }
+        CK(cudaMemsetAsync(h->fb.G[0], 0, sizeof(float4) * (size_t)h->P.n * h->P.n * h->P.n, st));
+        launch_p2g_scatter(P, h->fb.P[0], h->fb.vc, n, h->fb.G[0], h->fb.ctrl, h->elem_grid, st);
+        launch_grid_update_dense(P, h->fb.G[0], fr, h->elem_grid, st);
+        launch_g2p_split(P, h->fb.P[0], h->fb.vc, n, h->fb.G[0], h->fb.ctrl, h->elem_grid, st);
     }
     CK(cudaGetLastError());
     return MPM_OK;
 }
 
 mpm_status run_chunk(mpm_handle *h, int nsub, bool write_vc_last) {
-    if (!h->use_graphs) return issue_substeps(h, nsub, write_vc_last, h->stream);
+    // one or two launches need no graph
+    if (!h->use_graphs || (is_fused(h) && fused_many_steps(h->kernel_config))) return issue_substeps(h, nsub, write_vc_last, h->stream);
     // graphs are keyed by length, the vc flag, the tool-frame stride and the kernel configuration
     const std::pair<int, int> key(nsub, (write_vc_last ? 1 : 0) | (h->tstride << 1) | (h->kernel_config << 8));
     auto it = h->graphs.find(key);
@@ -1356,19 +1358,21 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
         tp.n = n;
         tp.ck = ck;
         const int c_last = (nck - 1) * ck, b_last = (nck - 1) % tp.nbuf;
-        for (int k = 0; k < n_substeps; ++k) {
+        for (int k = 0; k < n_substeps;) {
             if (k % ck == 0) id_image(h, tp.ckpt + (size_t)(k / ck) * tp.image);
+            int m = 1;
             if (k >= c_last) {
                 launch_fused_step_record(h->P, h->fb, tp.frames + (size_t)k * nt, step_record(h, k - c_last, b_last),
                                          record_grid(h), h->stream);
             } else {
                 // the configuration the reverse pass replays segments with, so that the
                 // replay follows the recorded trajectory up to the order of float atomics
-                const bool wv = (k + 1) % ck == 0;
-                launch_fused_step(h->P, h->fb, tp.frames + (size_t)k * nt, wv, record_grid(h), kRecordConfig,
-                                  h->stream);
+                m = std::min(ck, n_substeps - k);
+                launch_fused_steps(h->P, h->fb, tp.frames + (size_t)k * nt, m, true, record_grid(h), kRecordConfig,
+                                   h->stream);
             }
-            h->step += 1u;
+            h->step += (uint32_t)m;
+            k += m;
         }
         // the last sub-step kept v and C in its record, by output position: they
         // become the live state's

@@ -16,6 +16,7 @@ enum : uint32_t {
     kErrDomain = 2u,     // stencil clamped to the grid
     kErrCapacity = 4u,   // run-table or particle-count overflow
     kErrCfl = 8u,        // particle moved by more than one block in a sub-step
+    kErrStall = 16u,     // the CTAs of a launch of several sub-steps lost one another
 };
 
 // Per-environment material, in a device table indexed by environment.
@@ -84,7 +85,7 @@ struct Chunk {
     uint2 run[27];
 };
 // Per source block: which chunks it wrote in the last sub-step.
-struct BlockTab {
+struct __align__(16) BlockTab {
     uint32_t stamp;   // sub-step index the entry is valid for
     uint32_t first;   // first chunk index
     uint32_t npass;   // number of chunks
@@ -99,20 +100,23 @@ struct Ctrl {
     uint32_t n_particles;
     uint32_t err;               // sticky error bits
     uint32_t pad0[29];
-    uint32_t done;              // CTAs finished in the current fused launch
+    uint32_t done;              // arrivals of CTAs at the ends of the current launch's sub-steps
     uint32_t pad1[31];
-    uint32_t work;              // next work item of the current fused launch
-    uint32_t pad2[31];
-    uint32_t part_alloc;        // particle slots handed out in the current launch
-    uint32_t pad3[31];
-    uint32_t chunk_alloc;       // chunk entries handed out in the current launch
-    uint32_t pad4[31];
-    // active-block list sizes by sub-step parity: [0] heavy blocks, listed from
-    // the front, [1] light blocks, listed from the back (one 64-bit read)
-    uint32_t nactive[2][2];
-    uint32_t pad5[28];
-    uint32_t nclear[3];         // grid clear-list sizes, by sub-step mod 3
-    uint32_t pad6[29];
+    // Counters of a sub-step, by its index modulo their number: one slot is in
+    // use, and one that no CTA reads any more is returned to zero meanwhile, so
+    // that nothing is left to do between two sub-steps of a launch.
+    uint32_t work[3];           // next work item
+    uint32_t pad2[29];
+    uint32_t part_alloc[3];     // particle slots handed out
+    uint32_t pad3[29];
+    uint32_t chunk_alloc[3];    // chunk entries handed out
+    uint32_t pad4[29];
+    // active-block list sizes: [0] heavy blocks, listed from the front, [1]
+    // light blocks, listed from the back (one 64-bit read)
+    uint32_t nactive[3][2];
+    uint32_t pad5[26];
+    uint32_t nclear[4];         // clear-list sizes, by index of the grid they clear
+    uint32_t pad6[28];
 };
 static_assert(sizeof(Ctrl) == 7 * 128, "Ctrl: one 128-byte line per counter group");
 

@@ -32,9 +32,12 @@
 //
 // G2P and P2G run their x/y (and z/mass) components on the packed f32x2 pipe.
 //
+// A launch does one sub-step, or several with a grid-wide wait between them.
+//
 // Grid buffers rotate over three slots (read G_k, write G_{k+1}, clear
-// G_{k-1} for reuse), particle buffers and run tables over two; the last CTA
-// to finish resets the per-launch counters and advances the sub-step index.
+// G_{k-1} for reuse), particle buffers and run tables over two, counters over
+// three or four (a slot no CTA reads any more is zeroed meanwhile); the last CTA
+// of a launch advances the sub-step index.
 #include "common.cuh"
 #include "launch.h"
 
@@ -42,6 +45,7 @@ namespace gbmpm {
 
 namespace {
 
+constexpr uint32_t kMaxPolls = 1u << 22;   // of the wait between sub-steps: a few seconds
 constexpr int CMAX = 512;      // run candidates (source chunk x direction) per block
 constexpr float kFix = 4194304.0f;      // 2^22
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: float -> nearest int for |v| < 2^22
@@ -89,6 +93,9 @@ struct FusedSmem {
     static constexpr int NWP = NW <= 4 ? 4 : NW;
     alignas(16) uint8_t wcnt[2][28][NWP];
     uint32_t ncand, total, out_base, chunk_first, npass, mask, bmax, wide;
+    uint32_t nact, nheavy;         // active blocks, heavy ones among them
+    uint32_t m3;                   // sub-step index mod 3
+    bool go;                       // the launch's next sub-step may start
 };
 
 // resident CTAs per SM for which a configuration is compiled: 228 KB of shared
@@ -101,12 +108,20 @@ static_assert(5 * (sizeof(FusedSmem<128, 1>) + 1024) <= 228 * 1024, "shared memo
 static_assert(4 * (sizeof(FusedSmem<128, 2, 2>) + 1024) <= 228 * 1024, "configuration 2: four CTAs per SM");
 static_assert(2 * (sizeof(FusedSmem<256, 2, 2>) + 1024) <= 228 * 1024, "configuration 4: two CTAs per SM");
 
+__device__ __forceinline__ BlockTab load_tab(const BlockTab *p) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
+    BlockTab t;
+    t.stamp = v.x; t.first = v.y; t.npass = v.z; t.pad = v.w;
+    return t;
+}
+
 __device__ __forceinline__ int dir_dx(int d) { return d % 3 - 1; }
 __device__ __forceinline__ int dir_dy(int d) { return (d / 3) % 3 - 1; }
 __device__ __forceinline__ int dir_dz(int d) { return d / 9 - 1; }
 
+// list grid block g among those to clear of G_{stamp}, kept in list slot stamp mod 3
 __device__ __forceinline__ void mark_clear(const FusedBufs &B, uint32_t g, uint32_t stamp, int slot) {
-    if (atomicExch(&B.gstamp[g], stamp) != stamp) B.clist[slot][atomicAdd(&B.ctrl->nclear[slot], 1u)] = g;
+    if (atomicExch(&B.gstamp[g], stamp) != stamp) B.clist[slot][atomicAdd(&B.ctrl->nclear[stamp & 3u], 1u)] = g;
 }
 
 // nearest integer of v (|v| < 2^22) via the float mantissa
@@ -203,18 +218,20 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 // block's output was allocated) with their input positions, the list of
 // blocks in work order with each one's range, the list's length, and the grid
 // of each block's region before and after the grid operation.
-template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, bool RECORD = false, int PD = 1>
-__global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B,
-                                                                     const ToolFrame *__restrict__ tools,
-                                                                     StepRecord rec) {
+// One sub-step.  first: the launch's first (the arena is cleared then); last: the
+// launch's last (WRITE_VC: the one that writes v and C).  target: CTAs of the
+// launch times its sub-steps up to this one.  Returns whether to go on: false
+// after the last sub-step, or when the wait for the other CTAs ran out.
+template <bool WRITE_VC, int T, int GP, int MINB, bool RECORD, int PD>
+__device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const DevParams &P, const FusedBufs &B,
+                                              const ToolFrame *__restrict__ tools, const StepRecord &rec,
+                                              uint32_t step, uint32_t target, bool first, bool last) {
     using Smem = FusedSmem<T, GP, PD>;
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
     constexpr int NW = Smem::NW, GROUP = Smem::GROUP;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem &s = *reinterpret_cast<Smem *>(smem_raw);
+    constexpr bool kEarly = T * MINB <= 512;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     Ctrl *ctrl = B.ctrl;
-    const uint32_t step = *(volatile uint32_t *)&ctrl->step;
     const int par = step & 1, m3 = step % 3;
     const int m3n = (m3 + 1) % 3, m3c = (m3 + 2) % 3;
     // the two buffers of each array lie in one allocation: the sub-step's parity
@@ -227,13 +244,13 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     float4 *Gclr = B.G[m3c];
     // the active blocks: heavy ones listed from the front, light ones from the
     // back, and handed out heavy first so that the launch ends on short items
-    const unsigned long long nhl = *(volatile unsigned long long *)&ctrl->nactive[par][0];
+    const unsigned long long nhl = *(volatile unsigned long long *)&ctrl->nactive[m3][0];
     const uint32_t nheavy = (uint32_t)nhl, nact = (uint32_t)nhl + (uint32_t)(nhl >> 32);
     const uint32_t acap = B.nblocks;
     auto item_block = [&](uint32_t it) -> uint32_t {
-        return it >= nact ? 0u : B.alist[0][blk_in + (it < nheavy ? it : acap - 1u - (it - nheavy))];
+        return it >= s.nact ? 0u : __ldcg(&B.alist[0][blk_in + (it < s.nheavy ? it : acap - 1u - (it - s.nheavy))]);
     };
-    const uint32_t nclr = *(volatile uint32_t *)&ctrl->nclear[m3c];
+    const uint32_t nclr = *(volatile uint32_t *)&ctrl->nclear[(step + 3u) & 3u];     // G_{k-1}'s
     const uint32_t *__restrict__ clr = B.clist[m3c];
     const uint32_t nparticles = ctrl->n_particles;
     const uint32_t nchunk_cap = B.nblocks + nparticles / T + 1;
@@ -241,27 +258,46 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     const uint32_t nbe = P.nbe;
     uint32_t err = 0;
 
-    // prologue: work item blockIdx.x first (the shared counter hands out items
-    // gridDim.x, gridDim.x + 1, ... afterwards) and its inputs
+    // prologue: this CTA's first work item and its inputs (the shared counter hands
+    // out items gridDim.x, gridDim.x + 1, ... afterwards).
+    // The first gridDim.x items are the front of the heavy list, then the light
+    // list's, each CTA's at a place that does not depend on the lists' sizes: both
+    // entries are read together with the sizes.
+    if (tid == 0) { s.m3 = (uint32_t)m3; s.nact = nact; s.nheavy = nheavy; }
     if (tid == T - 1) {
-        const uint32_t it = blockIdx.x;
-        s.items[0] = it;
-        s.bids[0] = item_block(it);
+        const uint32_t back = gridDim.x - 1u - blockIdx.x;     // this CTA's place in the light list
+        const uint32_t *al = B.alist[0] + blk_in;
+        const uint32_t hb = blockIdx.x < acap ? __ldcg(&al[blockIdx.x]) : 0u;
+        const uint32_t lb = back < acap ? __ldcg(&al[acap - 1u - back]) : 0u;
+        const bool heavy = blockIdx.x < nheavy;
+        s.items[0] = heavy ? blockIdx.x : nheavy + back;
+        s.bids[0] = heavy ? hb : lb;
     }
     __syncthreads();
     if (s.items[0] < nact) prefetch_block<T>(s, 0, s.bids[0], B.inbox[0], blk_in, Gcur, P, tools, tid);
     // the P2G arena starts at zero; every flush returns the nodes it read to zero
-    for (int q = tid; q < 4 * kArena; q += T) (&s.acc[0][0])[q] = 0;
+    if (first)
+        for (int q = tid; q < 4 * kArena; q += T) (&s.acc[0][0])[q] = 0;
     // 0. while the first block's inputs land: clear the grid blocks G_{k-1} touched,
     //    so that sub-step k+1 can scatter into it (a different buffer from G_k)
     for (uint32_t q = blockIdx.x * T + tid; q < nclr * 64u; q += gridDim.x * T)
-        Gclr[clr[q >> 6] * 64u + (q & 63u)] = make_float4(0.f, 0.f, 0.f, 0.f);
+        Gclr[__ldcg(&clr[q >> 6]) * 64u + (q & 63u)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the counters that the next sub-step takes, idle since the last one but one
+    if (blockIdx.x == gridDim.x - 1 && tid == 0) {
+        if (!first && *(volatile uint32_t *)&ctrl->part_alloc[m3c] != nparticles) err |= kErrCapacity;
+        ctrl->work[m3n] = 0;
+        ctrl->part_alloc[m3n] = 0;
+        ctrl->chunk_alloc[m3n] = 0;
+        ctrl->nactive[m3c][0] = 0;
+        ctrl->nactive[m3c][1] = 0;
+        ctrl->nclear[(step + 2u) & 3u] = 0;
+    }
     cp_async_wait_all();
     __syncthreads();
 
     for (int cb = 0;; cb ^= 1) {
         const uint32_t item = s.items[cb];
-        if (item >= nact) break;
+        if (item >= s.nact) break;
         const uint32_t b = s.bids[cb];                 // global block
         if (RECORD && tid == 0) rec.act[item] = b;
         const uint32_t env = b >> (3 * P.lnb);          // environment
@@ -273,7 +309,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
         // the next work item: the atomic is issued here and its result is
         // consumed after this thread's share of the grid operation
         uint32_t next_item = 0;
-        if (tid == T - 1) next_item = gridDim.x + atomicAdd(&ctrl->work, 1u);
+        if (tid == T - 1) next_item = gridDim.x + atomicAdd(&ctrl->work[s.m3], 1u);
         uint32_t alloc_ob = 0, alloc_cf = 0;     // thread 0: the block's output range and chunks
         float4 *gv = s.graw[cb];
 
@@ -340,7 +376,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     const int d = 26 - lane;
                     const int sx = bx - dir_dx(d), sy = by - dir_dy(d), sz = bz - dir_dz(d);
                     if (sx >= 0 && sy >= 0 && sz >= 0 && sx < nb && sy < nb && sz < nb) {
-                        const BlockTab t = B.tabs[0][blk_in + eb0 + block_id(sx, sy, sz, nb)];
+                        const BlockTab t = load_tab(&B.tabs[0][blk_in + eb0 + block_id(sx, sy, sz, nb)]);
                         if (t.stamp == step) { np = t.npass; first = t.first; }
                     }
                 }
@@ -359,7 +395,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     if (c < ncand) {
                         int l = 0;
                         while (l < 26 && s.lane_off[l + 1] <= c) ++l;
-                        r = B.chunks[0][chunk_in + s.lane_first[l] + (c - s.lane_off[l])].run[26 - l];
+                        r = __ldcg(&B.chunks[0][chunk_in + s.lane_first[l] + (c - s.lane_off[l])].run[26 - l]);
                     }
                     uint32_t incl2 = r.y;
                     for (int o = 1; o < 32; o <<= 1) {
@@ -378,8 +414,8 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 s.total = carry;
                 s.npass = (carry + T - 1) / T;
                 // issued here, consumed after the barrier below
-                alloc_ob = atomicAdd(&ctrl->part_alloc, carry);
-                alloc_cf = atomicAdd(&ctrl->chunk_alloc, (carry + T - 1) / T);
+                alloc_ob = atomicAdd(&ctrl->part_alloc[s.m3], carry);
+                alloc_cf = atomicAdd(&ctrl->chunk_alloc[s.m3], (carry + T - 1) / T);
                 s.mask = 0;
                 s.bmax = 0;
                 s.wide = 0;
@@ -415,10 +451,39 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
             if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)(T + tid), tid, 1);
             cp_async_commit();
         }
-        if (s.items[cb ^ 1] < nact) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
+        if (s.items[cb ^ 1] < s.nact) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
         else cp_async_commit();
         const int ox = 4 * bx - 1, oy = 4 * by - 1, oz = 4 * bz - 1;   // arena origin
 
+        // Blocks of the next sub-step (the last warp) and grid blocks to clear before
+        // G_{k+1}'s reuse (the one before it): two chains of dependent global atomics.
+        // Where registers allow (kEarly) the stamps are exchanged before the last
+        // scatter and the lists appended to after the last flush, so that the first
+        // round trip is off the block's chain; otherwise both run after the block,
+        // beside warp 0's set-up of the next one.
+        uint32_t mark_b = 0, mark_old = step + 1;
+        auto mark_begin = [&](uint32_t mask) {
+            if (warp < NW - 2 || lane >= 27) return;
+            const int tx = bx + dir_dx(lane), ty = by + dir_dy(lane), tz = bz + dir_dz(lane);
+            if (tx < 0 || ty < 0 || tz < 0 || tx >= nb || ty >= nb || tz >= nb) return;
+            mark_b = eb0 + block_id(tx, ty, tz, nb);
+            if (warp == NW - 2) mark_old = atomicExch(&B.gstamp[mark_b], step + 1);
+            else if ((mask >> lane) & 1u) mark_old = atomicExch(&B.astamp[mark_b], step + 1);
+        };
+        auto mark_end = [&]() {
+            if (mark_old == step + 1) return;
+            if (warp == NW - 2) {
+                B.clist[(step + 1u) % 3u][atomicAdd(&ctrl->nclear[(step + 1) & 3u], 1u)] = mark_b;
+            } else {
+                // heavy: b itself (lane 13) with more particles now than one pass of the
+                // CTA takes.  A neighbour's mark wins only for blocks that particles
+                // enter from outside, which are light.
+                if (lane == 13 && total > (uint32_t)T)
+                    B.alist[0][blk_out + atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][0], 1u)] = mark_b;
+                else
+                    B.alist[0][blk_out + acap - 1u - atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][1], 1u)] = mark_b;
+            }
+        };
         for (uint32_t pass = 0; pass < npass; ++pass) {
             const uint32_t j = pass * T + tid;
             const bool valid = j < total;
@@ -579,7 +644,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                         }
                     for (int c = 0; c < 8; ++c) {
                         const int gi = (hx + 2 * (c & 1)) >> 2, gj = (hy + (c & 2)) >> 2, gk = (hz + ((c >> 1) & 2)) >> 2;
-                        mark_clear(B, eb0 + block_id(gi, gj, gk, nb), step + 1, m3n);
+                        mark_clear(B, eb0 + block_id(gi, gj, gk, nb), step + 1, (step + 1u) % 3u);
                     }
                 }
                 // --- destination block of the new state
@@ -673,7 +738,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 B.P[0].f0[out_off + pos] = make_float4(Fn[0], Fn[1], Fn[2], Fn[3]);
                 B.P[0].f1[out_off + pos] = make_float4(Fn[4], Fn[5], Fn[6], Fn[7]);
                 B.P[0].f2[out_off + pos] = Fn[8];
-                if (WRITE_VC) store_vc(B.vc, pos, vx, vy, vz, Cm);
+                if (WRITE_VC && last) store_vc(B.vc, pos, vx, vy, vz, Cm);
             }
 
             // --- P2G of the staged group (after every GP-th pass and the last one).
@@ -705,6 +770,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                     if (mine) s.order[off + (key >> 5)] = (uint16_t)sl;
                 }
                 __syncthreads();
+                if (kEarly && pass + 1 == npass) mark_begin(s.mask);
                 const uint32_t rows = (nin + 31u) >> 5;
                 for (uint32_t jr = warp; jr < rows; jr += NW) {
                     const uint32_t pos = lane * rows + jr;
@@ -780,6 +846,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                         s.acc[0][a] = 0; s.acc[1][a] = 0; s.acc[2][a] = 0; s.acc[3][a] = 0;
                     }
                 }
+                if (kEarly && pass + 1 == npass) mark_end();
                 // every thread read s.bmax, s.wide and the bucket sizes before the barriers
                 // above; the next group's atomics come after the barrier below
                 if (tid == 0) { s.bmax = 0; s.wide = 0; }
@@ -787,67 +854,120 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
                 __syncthreads();
             }
         }
-        // the block's direction mask and size, read before warp 0 reuses them for the
-        // next block
-        const uint32_t mask_b = s.mask, total_b = s.total;
+        const uint32_t mask_b = s.mask;     // before warp 0 takes it for the next block
         cp_async_wait_all();
         __syncthreads();
-        // blocks of the next sub-step (the last warp) and grid blocks to clear before
-        // G_{k+1}'s reuse (the one before it): two chains of dependent global atomics
-        // that run beside warp 0's set-up of the next block
-        if (warp >= NW - 2 && lane < 27) {
-            const int tx = bx + dir_dx(lane), ty = by + dir_dy(lane), tz = bz + dir_dz(lane);
-            if (tx >= 0 && ty >= 0 && tz >= 0 && tx < nb && ty < nb && tz < nb) {
-                const uint32_t tb = eb0 + block_id(tx, ty, tz, nb);
-                if (warp == NW - 1 && ((mask_b >> lane) & 1u)) {
-                    // heavy: b itself (lane 13) with more particles now than one pass
-                    // of the CTA takes.  A neighbour's mark wins only for blocks that
-                    // particles enter from outside, which are light.
-                    if (atomicExch(&B.astamp[tb], step + 1) != step + 1) {
-                        if (lane == 13 && total_b > (uint32_t)T)
-                            B.alist[0][blk_out + atomicAdd(&ctrl->nactive[par ^ 1][0], 1u)] = tb;
-                        else
-                            B.alist[0][blk_out + acap - 1u - atomicAdd(&ctrl->nactive[par ^ 1][1], 1u)] = tb;
-                    }
-                }
-                if (warp == NW - 2) mark_clear(B, tb, step + 1, m3n);
-            }
+        if (!kEarly || npass == 0) {
+            mark_begin(mask_b);
+            mark_end();
         }
     }
 
     if (err) atomicOr(&ctrl->err, err);
-    // last CTA: reset per-launch counters, advance the sub-step
     __syncthreads();
-    // No fence before the done counter: the last CTA reads only part_alloc,
-    // whose atomics every CTA consumed (its block's output range) before
-    // counting itself done, and everything it writes is read by the next
-    // launch, after this one has completed.
-    if (tid == 0) {
-        const uint32_t prev = atomicAdd(&ctrl->done, 1u);
-        if (prev == gridDim.x - 1) {
+    // Arrivals count up over the launch's sub-steps, target = CTAs x sub-steps so
+    // far.  At the end of the launch's last one no fence: the last CTA reads only
+    // part_alloc, whose atomics every CTA consumed (its block's output range)
+    // before it arrived, and what it writes is read by the next launch.
+    // Elsewhere the arrival releases this CTA's writes and the wait acquires the
+    // others'.
+    if (last) {
+        if (tid == 0 && atomicAdd(&ctrl->done, 1u) == target - 1u) {
             __threadfence();
-            if (*(volatile uint32_t *)&ctrl->part_alloc != nparticles) atomicOr(&ctrl->err, kErrCapacity);
-            ctrl->work = 0;
-            ctrl->part_alloc = 0;
-            ctrl->chunk_alloc = 0;
-            ctrl->nactive[par][0] = 0;
-            ctrl->nactive[par][1] = 0;
-            ctrl->nclear[m3c] = 0;
+            if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
             ctrl->done = 0;
             if (RECORD) *rec.nact = nact;
             ctrl->step = step + 1;
         }
+        return false;
+    }
+    if (tid == 0) {
+        // every CTA is resident (cooperative launch), so the wait ends when the last
+        // one arrives; after some seconds it ends with an error
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctrl->done) : "memory");
+        uint32_t now, polls = 0;
+        do {
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&ctrl->done) : "memory");
+        } while (now < target && ++polls < kMaxPolls);
+        asm volatile("fence.acq_rel.gpu;" ::: "memory");
+        if (now < target) atomicOr(&ctrl->err, kErrStall);
+        s.go = now >= target;
+    }
+    __syncthreads();
+    return s.go;
+}
+
+// Launches of several sub-steps where the registers allow it.  A small scene's
+// sub-step is one block's chain of round trips plus the launch gap and the ramp
+// of its CTAs; without the latter two, and with the neighbour marks begun before
+// the last scatter, the 30K slab takes 13.8 instead of 16.5 us per sub-step of a
+// 25-sub-step frame (256 threads, 2 CTAs per SM) and the 8K cube 22.4 -> 21.8.  At 80
+// registers a thread the loop's state spills: 1M particles 94.6 -> 106 us.
+template <int T, int MINB>
+constexpr bool kManySteps = T * MINB <= 640;
+
+// nsub sub-steps, the tool frames of each `frames` entries after the one
+// before.  One launch for all of them spares the launch gap and the ramp of the
+// CTAs between sub-steps; the CTAs then wait for one another, so nsub > 1 needs
+// a cooperative launch.  v and C are written by the last one (if WRITE_VC).
+template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, bool RECORD = false, int PD = 1>
+__global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B,
+                                                        const ToolFrame *__restrict__ tools, uint32_t frames,
+                                                        StepRecord rec, uint32_t nsub) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FusedSmem<T, GP, PD> &s = *reinterpret_cast<FusedSmem<T, GP, PD> *>(smem_raw);
+    const uint32_t step = *(volatile uint32_t *)&B.ctrl->step;
+    if constexpr (!kManySteps<T, MINB> || RECORD) {
+        fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools, rec, step, gridDim.x, true, true);
+    } else {
+        for (uint32_t k = 0;; ++k)
+            if (!fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools + (size_t)k * frames, rec, step + k,
+                                                                  (k + 1) * gridDim.x, k == 0, k + 1 == nsub))
+                break;
     }
 }
 
+// nsub sub-steps as one launch, cooperative if there are several, or one by one
+// where the CTAs cannot all be resident (a context with a part of the SMs).
+template <typename Kernel>
+void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, const FusedBufs &B, const ToolFrame *tools,
+                  const StepRecord &rec, int nsub, int grid, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = nsub > 1 ? 1 : 0;
+    const uint32_t frames = (uint32_t)(P.n_envs * P.tstride);
+    // a failure is left for cudaGetLastError
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P, B, tools, frames, rec, (uint32_t)nsub);
+    if (nsub > 1 && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
+        cudaGetLastError();
+        cfg.numAttrs = 0;
+        for (int k = 0; k < nsub; ++k)
+            cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, rec, 1u);
+    }
+}
+
+// With 128 registers the variant that writes v and C does not spill either, and
+// all sub-steps are one launch; otherwise the last is its own.
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
-void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, bool write_vc, int grid,
+void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc, int grid,
                     cudaStream_t st) {
+    constexpr bool kOne = T * MINB <= 512;
+    const size_t smem = sizeof(FusedSmem<T, GP, PD>), frames = (size_t)P.n_envs * P.tstride;
     const StepRecord none{};
-    if (write_vc)
-        k_fused_step<true, T, GP, MINB, false, PD><<<grid, T, sizeof(FusedSmem<T, GP, PD>), st>>>(P, B, tools, none);
-    else
-        k_fused_step<false, T, GP, MINB, false, PD><<<grid, T, sizeof(FusedSmem<T, GP, PD>), st>>>(P, B, tools, none);
+    const int plain = !write_vc ? nsub : kOne ? 0 : nsub - 1;
+    const int per = kManySteps<T, MINB> ? plain : 1;
+    for (int k = 0; k < plain; k += per)
+        launch_steps(k_fused_step<false, T, GP, MINB, false, PD>, T, smem, P, B, tools + k * frames, none, per, grid, st);
+    if (plain < nsub)
+        launch_steps(k_fused_step<true, T, GP, MINB, false, PD>, T, smem, P, B, tools + plain * frames, none,
+                     nsub - plain, grid, st);
 }
 
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
@@ -863,16 +983,18 @@ int variant_occupancy() {
 
 }  // namespace
 
-void launch_fused_step(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, bool write_vc, int grid,
-                       int config, cudaStream_t st) {
+void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc,
+                        int grid, int config, cudaStream_t st) {
     switch (config) {
-    case 1: launch_variant<256, 1>(P, B, tools, write_vc, grid, st); break;
-    case 2: launch_variant<128, 2, kMinBlocks<128, 2>, 2>(P, B, tools, write_vc, grid, st); break;
-    case 3: launch_variant<128, 1>(P, B, tools, write_vc, grid, st); break;
-    case 4: launch_variant<256, 2, 2, 2>(P, B, tools, write_vc, grid, st); break;   // 2 CTAs per SM, 128 registers
-    default: launch_variant<256, 2>(P, B, tools, write_vc, grid, st); break;
+    case 1: launch_variant<256, 1>(P, B, tools, nsub, write_vc, grid, st); break;
+    case 2: launch_variant<128, 2, kMinBlocks<128, 2>, 2>(P, B, tools, nsub, write_vc, grid, st); break;
+    case 3: launch_variant<128, 1>(P, B, tools, nsub, write_vc, grid, st); break;
+    case 4: launch_variant<256, 2, 2, 2>(P, B, tools, nsub, write_vc, grid, st); break;   // 2 CTAs per SM, 128 registers
+    default: launch_variant<256, 2>(P, B, tools, nsub, write_vc, grid, st); break;
     }
 }
+
+bool fused_many_steps(int config) { return config != 0 && config != 1; }
 
 int fused_step_threads(int config) { return config == 2 || config == 3 ? 128 : 256; }
 
@@ -888,7 +1010,7 @@ int fused_record_occupancy() {
 
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
                               int grid, cudaStream_t st) {
-    k_fused_step<false, 256, 2, 2, true><<<grid, 256, sizeof(FusedSmem<256, 2>), st>>>(P, B, tools, rec);
+    launch_steps(k_fused_step<false, 256, 2, 2, true>, 256, sizeof(FusedSmem<256, 2>), P, B, tools, rec, 1, grid, st);
 }
 
 // Also opts the kernel into its dynamic shared memory size on the current

@@ -217,14 +217,14 @@ __global__ void k_init_tables(DevParams P, const uint32_t *__restrict__ offsets,
         for (int d = 0; d < 27; ++d) ch.run[d] = make_uint2(d == 13 ? off : 0u, d == 13 ? c : 0u);
         B.inbox[par][(size_t)b * kInbox + 13 * kNpMax] = make_uint4(off, c, step, 0u);
         B.astamp[b] = step;
-        B.alist[par][atomicAdd(&B.ctrl->nactive[par][0], 1u)] = b;
+        B.alist[par][atomicAdd(&B.ctrl->nactive[m3][0], 1u)] = b;
         const uint32_t e = b / P.nbe, bl = b % P.nbe;
         const int bx = bl % P.nb, by = (bl / P.nb) % P.nb, bz = bl / (P.nb * P.nb);
         for (int d = 0; d < 27; ++d) {
             const int sx = bx + d % 3 - 1, sy = by + (d / 3) % 3 - 1, sz = bz + d / 9 - 1;
             if (sx < 0 || sy < 0 || sz < 0 || sx >= P.nb || sy >= P.nb || sz >= P.nb) continue;
             const uint32_t g = e * P.nbe + block_id(sx, sy, sz, P.nb);
-            if (atomicExch(&B.gstamp[g], step) != step) B.clist[m3][atomicAdd(&B.ctrl->nclear[m3], 1u)] = g;
+            if (atomicExch(&B.gstamp[g], step) != step) B.clist[m3][atomicAdd(&B.ctrl->nclear[step & 3u], 1u)] = g;
         }
     }
 }

@@ -176,9 +176,13 @@ struct ReverseArgs {
 // config (MPM_KERNEL_*): 0 = 256 threads, 2 passes per P2G flush; 1 = 256, 1;
 // 2 = 128, 2; 3 = 128, 1; 4 = 256, 2 with 2 CTAs per SM.  Configurations 2 and
 // 4 copy each pass's particles two passes ahead, the others one pass ahead.
-void launch_fused_step(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, bool write_vc, int grid,
-                       int config, cudaStream_t st);
+// nsub sub-steps with the frame tables at tools (n_envs tstride entries each),
+// the last of which also writes v and C if write_vc.  grid: at most the number
+// of CTAs that are resident at once.
+void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc,
+                        int grid, int config, cudaStream_t st);
 int fused_step_occupancy(int config);
+bool fused_many_steps(int config);     // whether a launch takes many sub-steps
 int fused_step_threads(int config);
 int fused_record_occupancy();
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
