@@ -263,7 +263,7 @@ mpm_status mpm_extract_surface(mpm_handle *h, int32_t env, float iso, float *tri
  * of a block when there are few blocks per CTA.  Not in the paper (its
  * Taichi kernels are tuned by Taichi); a utility of this library. */
 enum {
-    MPM_KERNEL_T256_G2 = 0, /* 256 threads, 512 particles per flush (the default) */
+    MPM_KERNEL_T256_G2 = 0, /* 256 threads, 512 particles per flush */
     MPM_KERNEL_T256_G1 = 1, /* 256 threads, 256 particles per flush */
     MPM_KERNEL_T128_G2 = 2, /* 128 threads, 256 particles per flush, particles copied 2 passes ahead */
     MPM_KERNEL_T128_G1 = 3, /* 128 threads, 128 particles per flush */
@@ -272,17 +272,21 @@ enum {
 };
 
 /* Select the fused kernel configuration (fused pipeline; the split pipeline
- * ignores it).  MPM_ERR_ARG if out of range or not resident on this GPU. */
+ * ignores it).  Until one is selected, here or by mpm_autotune, every load takes
+ * one by the number of particles and their volume (which may also be one that
+ * cannot be selected: 512 threads, for small dense scenes).  MPM_ERR_ARG if
+ * out of range or not resident on this GPU. */
 mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config);
 
-/* The current configuration, its CTA size and the persistent grid size (CTAs
- * per launch); any output may be NULL. */
+/* The selected configuration (0 while none is), and the CTA size and the
+ * persistent grid size (CTAs per launch) in use; any output may be NULL. */
 mpm_status mpm_get_kernel_config(mpm_handle *h, int32_t *config, int32_t *threads, int32_t *ctas);
 
 /* Autotuner: time every configuration on the handle's own state (one
  * untimed call of n_substeps sub-steps, then three timed calls, each trial
  * starting from the same snapshot of the particles and tools), select the
- * one with the smallest median call time and restore the state as it was
+ * one with the smallest median call time (none, and best 0, where the load's
+ * own choice of 512 threads is faster) and restore the state as it was
  * (particle order inside the library may change; mpm_read_particles returns
  * the same values).  times_ms (MPM_KERNEL_CONFIGS floats: the median call
  * times, -1 for configurations that do not fit) and best may be NULL.  Needs a loaded fused-pipeline handle

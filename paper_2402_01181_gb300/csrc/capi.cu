@@ -123,7 +123,8 @@ struct mpm_handle {
     void *alloc_ctx = nullptr;
     std::vector<Alloc> allocs;
     int device = 0, num_sms = 0, fused_grid = 0, elem_grid = 0;
-    int kernel_config = 0;          // MPM_KERNEL_* of the fused sub-step
+    int kernel_config = 0;          // the fused sub-step's configuration in use
+    bool config_set = false;        // by the caller or the autotuner; otherwise by choose_config at each load
     int n_envs = 1;
     int sub_chunk = 512;        // sub-steps per captured graph / frame upload
     int tstride = 0;            // tool frames per environment in the uploaded table
@@ -632,6 +633,35 @@ mpm_status mpm_set_stream(mpm_handle *h, void *cuda_stream) {
 
 namespace {
 
+mpm_status apply_kernel_config(mpm_handle *h, int config);
+
+static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuration follows the selectable ones");
+// The fused sub-step's configuration for the loaded particles, where the caller
+// has set none.  By the number of filled 4x4x4 blocks, estimated as the particles
+// over a full block's number (64 cells' worth, from their volume) times 1.5, or
+// times 2 for sparse bodies, as the blocks at the surface are filled in part.
+// Measured on 152 SMs, us per sub-step under configurations 0, 2, 3, 4 and 5:
+// - as long as every block can have a CTA of its own, one block's chain counts, so
+//   the largest CTAs that fit (8K cube 21.7, 37, 43, 21.8, 18.1; 50K at 10 per cell
+//   17.8, 22.7, 25.6, 14.2, 12.8; 30K slab 17.1, 17.7, 21.4, 13.8, 17.5; 50K slab at
+//   3 per cell 17.0, 14.9, 18.7, 16.9, 19.5);
+// - beyond, sparse blocks waste the fewest threads of the smallest CTAs (200K slab
+//   47, 43, 39, 45, 61; 256 environments 1389, 1200, 1150, 1520, 2340), dense ones
+//   run from 4 to 5 blocks per CTA on with the most warps (500K at 8 per cell 51.4,
+//   59, 61, 50.5, 70; 800K 72.4, 81, 86, 76.3, 106; 1M 94, 105, 109, 100, 138).
+int choose_config(const mpm_handle *h) {
+    const double cell = 1.0 / ((double)h->P.n * h->P.n * h->P.n), sms = h->num_sms;
+    double full = 0.0;
+    for (int e = 0; e < h->n_envs; ++e)
+        full += (double)(h->env_off[e + 1] - h->env_off[e]) * h->env_vol[e] / (64.0 * cell);
+    const bool sparse = (double)h->n < 6.0 * 64.0 * full;
+    const double blocks = full * (sparse ? 2.0 : 1.5);
+    if (blocks <= sms) return kConfigT512;
+    if (blocks <= 2.0 * sms) return MPM_KERNEL_T256_G2_C2;
+    if (sparse) return blocks <= 4.0 * sms ? MPM_KERNEL_T128_G2 : MPM_KERNEL_T128_G1;
+    return blocks <= 9.0 * sms ? MPM_KERNEL_T256_G2_C2 : MPM_KERNEL_T256_G2;
+}
+
 // Replace the state of every environment: counts[e] particles of environment
 // e, stored env-major in x, v, F, C; volumes[e] its particle volume.
 mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const float *v, const float *F,
@@ -684,6 +714,10 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     h->step = k0;
     h->n = n;
     h->taken = 0;
+    if (is_fused(h) && !h->config_set) {
+        const int config = choose_config(h);
+        if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
+    }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
     if (is_fused(h)) {
         for (int g = 0; g < 3; ++g) CK(cudaMemsetAsync(h->fb.G[g], 0, sizeof(float4) * nn, h->stream));
@@ -1605,14 +1639,16 @@ extern "C" {
 mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config) {
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
-    if (config < 0 || config >= kFusedConfigs) return fail(MPM_ERR_ARG, "kernel configuration %d out of range", config);
-    return apply_kernel_config(h, config);
+    if (config < 0 || config >= MPM_KERNEL_CONFIGS) return fail(MPM_ERR_ARG, "kernel configuration %d out of range", config);
+    st = apply_kernel_config(h, config);
+    if (st == MPM_OK) h->config_set = true;
+    return st;
 }
 
 mpm_status mpm_get_kernel_config(mpm_handle *h, int32_t *config, int32_t *threads, int32_t *ctas) {
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
-    if (config) *config = h->kernel_config;
+    if (config) *config = h->config_set ? h->kernel_config : MPM_KERNEL_T256_G2;
     if (threads) *threads = fused_step_threads(h->kernel_config);
     if (ctas) *ctas = h->fused_grid;
     return MPM_OK;
@@ -1629,9 +1665,9 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
     if (n_substeps < 1) return fail(MPM_ERR_ARG, "n_substeps must be >= 1");
     if ((st = poll_error(h, true)) != MPM_OK) return st;
     if (times_ms)
-        for (int c = 0; c < kFusedConfigs; ++c) times_ms[c] = -1.f;
+        for (int c = 0; c < MPM_KERNEL_CONFIGS; ++c) times_ms[c] = -1.f;
     if (h->n == 0) {
-        if (best) *best = h->kernel_config;
+        if (best) *best = h->config_set ? h->kernel_config : MPM_KERNEL_T256_G2;
         return MPM_OK;
     }
     // snapshot of the state, the tools and the counters; every trial starts from it
@@ -1649,16 +1685,20 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
         vols[e] = (float)h->env_vol[e];
     }
     const int start = h->kernel_config;
+    const bool start_set = h->config_set;
     cudaEvent_t a = nullptr, b = nullptr;
     CK(cudaEventCreate(&a));
     CK(cudaEventCreate(&b));
+    h->config_set = true;     // the trials' loads keep the trial's configuration
     auto restore = [&]() -> mpm_status {
         h->tools = tools0;
         return load_impl(h, counts.data(), sx, sv, sF, sC, vols.data(), 1);
     };
     int pick = start;
     float best_ms = 3.0e38f;
-    for (int c = 0; c < kFusedConfigs && st == MPM_OK; ++c) {
+    // the selectable ones, and the library's own where a load would take it
+    const int last = choose_config(h) == kConfigT512 ? kConfigT512 : MPM_KERNEL_CONFIGS - 1;
+    for (int c = 0; c <= last && st == MPM_OK; ++c) {
         if (fused_step_occupancy(c) < 1) continue;
         if ((st = apply_kernel_config(h, c)) != MPM_OK) break;
         if ((st = restore()) != MPM_OK) break;
@@ -1678,17 +1718,19 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
         if (st != MPM_OK) break;
         std::sort(reps, reps + kTuneReps);
         const float ms = reps[kTuneReps / 2];
-        if (times_ms) times_ms[c] = ms;
+        if (times_ms && c < MPM_KERNEL_CONFIGS) times_ms[c] = ms;
         if (ms < best_ms) { best_ms = ms; pick = c; }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     mpm_status st2 = apply_kernel_config(h, st == MPM_OK ? pick : start);
+    if (st != MPM_OK) h->config_set = start_set;
+    else if (pick == kConfigT512) h->config_set = false;     // the load's choice again
     if (st2 == MPM_OK) st2 = restore();
     h->taken = taken0;
     if (st != MPM_OK) return st;
     if (st2 != MPM_OK) return st2;
-    if (best) *best = pick;
+    if (best) *best = h->config_set ? pick : MPM_KERNEL_T256_G2;
     return MPM_OK;
 }
 

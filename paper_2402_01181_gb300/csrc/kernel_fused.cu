@@ -101,7 +101,7 @@ struct FusedSmem {
 // resident CTAs per SM for which a configuration is compiled: 228 KB of shared
 // memory per SM with 1 KB reserved per CTA, 64 K registers
 template <int T, int GP>
-constexpr int kMinBlocks = T == 256 ? 3 : (GP == 1 ? 5 : 4);
+constexpr int kMinBlocks = T == 512 ? 1 : T == 256 ? 3 : (GP == 1 ? 5 : 4);
 static_assert(3 * (sizeof(FusedSmem<256, 2>) + 1024) <= 228 * 1024, "shared memory for three CTAs per SM");
 static_assert(4 * (sizeof(FusedSmem<128, 2>) + 1024) <= 228 * 1024, "shared memory for four CTAs per SM");
 static_assert(5 * (sizeof(FusedSmem<128, 1>) + 1024) <= 228 * 1024, "shared memory for five CTAs per SM");
@@ -990,13 +990,14 @@ void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame 
     case 2: launch_variant<128, 2, kMinBlocks<128, 2>, 2>(P, B, tools, nsub, write_vc, grid, st); break;
     case 3: launch_variant<128, 1>(P, B, tools, nsub, write_vc, grid, st); break;
     case 4: launch_variant<256, 2, 2, 2>(P, B, tools, nsub, write_vc, grid, st); break;   // 2 CTAs per SM, 128 registers
+    case 5: launch_variant<512, 2>(P, B, tools, nsub, write_vc, grid, st); break;         // 1 CTA per SM, 128 registers
     default: launch_variant<256, 2>(P, B, tools, nsub, write_vc, grid, st); break;
     }
 }
 
 bool fused_many_steps(int config) { return config != 0 && config != 1; }
 
-int fused_step_threads(int config) { return config == 2 || config == 3 ? 128 : 256; }
+int fused_step_threads(int config) { return config == 5 ? 512 : config == 2 || config == 3 ? 128 : 256; }
 
 // The recording sub-step of the differentiable rollout: the configuration of
 // 256 threads, 2 passes per flush and 2 CTAs per SM (128 registers).
@@ -1021,6 +1022,7 @@ int fused_step_occupancy(int config) {
     case 2: return variant_occupancy<128, 2, kMinBlocks<128, 2>, 2>();
     case 3: return variant_occupancy<128, 1>();
     case 4: return variant_occupancy<256, 2, 2, 2>();
+    case 5: return variant_occupancy<512, 2>();
     default: return variant_occupancy<256, 2>();
     }
 }

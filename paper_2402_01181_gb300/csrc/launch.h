@@ -174,8 +174,9 @@ struct ReverseArgs {
     uint32_t *touch_n;         // receives the number of work-list blocks (do_g2p)
 };
 // config (MPM_KERNEL_*): 0 = 256 threads, 2 passes per P2G flush; 1 = 256, 1;
-// 2 = 128, 2; 3 = 128, 1; 4 = 256, 2 with 2 CTAs per SM.  Configurations 2 and
-// 4 copy each pass's particles two passes ahead, the others one pass ahead.
+// 2 = 128, 2; 3 = 128, 1; 4 = 256, 2 with 2 CTAs per SM; 5 = 512, 2 with 1 CTA
+// per SM (chosen by the library only).  Configurations 2 and 4 copy each pass's
+// particles two passes ahead, the others one pass ahead.
 // nsub sub-steps with the frame tables at tools (n_envs tstride entries each),
 // the last of which also writes v and C if write_vc.  grid: at most the number
 // of CTAs that are resident at once.
@@ -187,7 +188,7 @@ int fused_step_threads(int config);
 int fused_record_occupancy();
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
                               int grid, cudaStream_t st);
-constexpr int kFusedConfigs = 5;
+constexpr int kConfigT512 = 5;          // beside the MPM_KERNEL_CONFIGS that a caller can select
 constexpr int kFusedMinThreads = 128;     // chunk tables are sized for the smallest CTA
 // Inbox of a block: entry d * kNpMax + p holds the run of source pass p
 // coming from direction d (source block = block - dir(d)); the last entry,

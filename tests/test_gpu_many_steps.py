@@ -1,0 +1,95 @@
+"""Several sub-steps per launch and the configuration a load chooses."""
+import numpy as np
+import pytest
+
+import helpers as H
+from oracle import oracle as O
+from paper_2402_01181_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+CHOSEN = None            # no configuration set: the load's choice
+
+
+@pytest.fixture(scope="module")
+def M():
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2402_01181_gb300 import mpm
+    return mpm
+
+
+@pytest.mark.parametrize("config", [CHOSEN, 0, 1, 2, 3, 4])
+def test_calls_of_several_lengths_follow_the_oracle(M, config):
+    """Calls of 1, 2, 5, 1 and 6 sub-steps (every buffer parity and counter slot
+    starts a launch and ends one): the 15 sub-steps within the bounds of 200
+    (x to 1e-3 dx, F to 1e-4), the order sorted by block after each call."""
+    sc = H.perturbed_scene(scenes.cube8k(3), seed=4)
+    sim = M.sim_from_scene(sc)
+    if config is not CHOSEN:
+        sim.set_kernel_config(config)
+    for k in (1, 2, 5, 1, 6):
+        sim.step(k)
+        ids, keys = sim.read_order()
+        x = sim.read()["x"]
+        assert np.array_equal(keys, O.block_keys(sc.n_grid, x)[ids]) and np.all(np.diff(keys.astype(np.int64)) >= 0)
+        assert np.array_equal(np.sort(ids), np.arange(sc.n))
+    out = sim.read()
+    sim.close()
+    st = O.State(sc.x, sc.v, sc.C, sc.F)
+    H.oracle_steps(sc, st, 0, 15)
+    assert np.abs(out["x"] - st.x).max() <= 1e-3 * sc.dx
+    assert np.abs(out["F"] - st.F).max() <= 1e-4
+
+
+@pytest.mark.parametrize("n,ppc,grid,threads,ctas_per_sm", [
+    (8192, 16.0, 32, 512, 1),        # 8 blocks' worth: a block's chain, the fewest passes
+    (30000, 3.18, 64, 256, 2),       # 147: a CTA for every block, no spills
+    (800000, 9.0, 128, 256, 3),      # 1389, dense
+    (50000, 3.2, 64, 128, 4),        # 244, sparse
+    (400000, 3.3, 128, 128, 5),      # 1894, sparse
+])
+def test_load_chooses_by_size_and_density(M, n, ppc, grid, threads, ctas_per_sm):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    x = (0.2 + 0.6 * np.random.default_rng(1).random((n, 3))).astype(np.float32)
+    cfg = M.make_config(grid, 1e-5, 1e4, 0.3, 1e3, max_particles=n)
+    sim = M.Sim(cfg)
+    sim.load(x, 1.0 / (ppc * grid ** 3))
+    got = sim.kernel_config()
+    assert got == {"config": 0, "threads": threads, "ctas": ctas_per_sm * sms}
+    sim.set_kernel_config(2)         # a set one is kept by later loads
+    sim.load(x, 1.0 / (ppc * grid ** 3))
+    assert sim.kernel_config()["config"] == 2 and sim.kernel_config()["threads"] == 128
+    sim.close()
+
+
+@pytest.mark.parametrize("count", [511, 512, 513, 1024, 1025, 4097])
+def test_512_threads_single_substep_parity(M, count):
+    """Blocks of one, two and more passes of 512 particles, and the run-table
+    path of more than four, under a moving capsule."""
+    rng = np.random.default_rng(count)
+    n = 32
+    x = (0.40625 + 0.125 * rng.random((count, 3))).astype(np.float32)
+    v, C, F = scenes.random_state(x, count, v_scale=0.3, c_scale=1.0, f_dev=0.05)
+    cap = scenes.capsule_shape(0.04, 0.05)
+    sc = scenes.Scene("blob", n_grid=n, dt=1e-4, E=2e3, nu=0.3, rho=1e3, x=x, particle_volume=2e-8, v=v, C=C, F=F,
+                      friction=0.3,
+                      tools=[scenes.Tool(cap, lambda s: np.array([0.47, 0.61 - 1e-4 * (s + 1), 0.46, 0.1, 0.0, 0.2]))])
+    sim = M.sim_from_scene(sc)
+    assert sim.kernel_config()["threads"] == 512
+    ids, _ = sim.read_order()
+    start = sim.read()
+    sim.set_tool(0, sc.tools[0].pose(0), sc.tools[0].shape)
+    sim.step(1)
+    out = sim.read()
+    ids2, _ = sim.read_order()
+    sim.close()
+    assert np.array_equal(ids2, O.sorted_order(O.block_keys(n, out["x"]), ids))
+    st = H.oracle_state(start)
+    mask = H.contact_mask_nodes(sc, st, 0)
+    skip = H.particles_touching(mask, st.x, n)
+    H.oracle_steps(sc, st, 0, 1, call_len=1)
+    assert mask.sum() <= 5
+    ok, errs = H.compare_particles(out, st, sc.dx, skip)
+    assert ok, errs
