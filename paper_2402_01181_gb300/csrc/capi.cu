@@ -147,6 +147,7 @@ struct mpm_handle {
     ToolFrame *h_frames[2] = {nullptr, nullptr};
     int frames_next = 0;
     uint32_t *h_err = nullptr;       // pinned copy of Ctrl::err
+    uint32_t *h_total = nullptr;     // pinned: number of triangles of a surface
     cudaEvent_t ev_err = nullptr, ev_frames[2] = {nullptr, nullptr};
     // the reverse pass's segment replays run on their own stream, one segment
     // ahead of the reverse sub-steps: rp_rec[b] marks record buffer b complete,
@@ -179,7 +180,7 @@ struct mpm_handle {
     float *tune_snap = nullptr;
     size_t tune_cap = 0;
     // surface extraction scratch
-    uint32_t *surf_counts = nullptr, *surf_sums = nullptr;
+    SurfaceScratch surf{};
     float *surf_tri = nullptr;
     size_t surf_tri_cap = 0;
 };
@@ -590,9 +591,10 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
         e = cudaMallocHost(&h->h_frames[b], sizeof(ToolFrame) * (size_t)h->sub_chunk * n_envs * MPM_MAX_TOOLS);
         if (e != cudaSuccess) return bail(fail(MPM_ERR_ALLOC, "cudaMallocHost: %s", cudaGetErrorString(e)));
     }
-    e = cudaMallocHost(&h->h_err, sizeof(uint32_t));
+    e = cudaMallocHost(&h->h_err, 2 * sizeof(uint32_t));
     if (e != cudaSuccess) return bail(fail(MPM_ERR_ALLOC, "cudaMallocHost: %s", cudaGetErrorString(e)));
     *h->h_err = 0;
+    h->h_total = h->h_err + 1;
     if ((e = cudaEventCreateWithFlags(&h->ev_err, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[0], cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[1], cudaEventDisableTiming)) != cudaSuccess ||
@@ -1750,38 +1752,39 @@ mpm_status mpm_extract_surface(mpm_handle *h, int32_t env, float iso, float *tri
     if (!std::isfinite(iso)) return fail(MPM_ERR_ARG, "non-finite iso");
     if (!h->loaded) return fail(MPM_ERR_STATE, "no particles loaded");
     const int n = h->P.n;
-    const size_t cells = (size_t)(n - 1) * (n - 1) * (n - 1);
-    const size_t nblk = (cells + 1 + 1023) / 1024;
-    if (!h->surf_counts) {
-        if ((st = dalloc_t(h, &h->surf_counts, cells + 1)) != MPM_OK) return st;
-        if ((st = dalloc_t(h, &h->surf_sums, nblk + 1)) != MPM_OK) return st;
+    const SurfaceSizes sz = surface_sizes(n);
+    if (!h->surf.sums) {
+        SurfaceScratch z{};
+        if ((st = dalloc_t(h, &z.bits, sz.bits)) != MPM_OK) return st;
+        if ((st = dalloc_t(h, &z.counts, sz.words)) != MPM_OK) return st;
+        if ((st = dalloc_t(h, &z.sums, sz.units + 1)) != MPM_OK) return st;
+        h->surf = z;
     }
     const float4 *G = current_grid(h);
     const double dx = 1.0 / n;
     const float scale = (float)(1.0 / (h->env_rho[env] * dx * dx * dx));   // density / rho
-    launch_surface_count_scan(G, n, h->P.nb, h->nbe, (uint32_t)env, scale, iso, h->surf_counts, h->surf_sums,
-                              h->elem_grid, h->stream);
+    launch_surface_count(G, n, h->P.nb, h->nbe, (uint32_t)env, scale, iso, h->surf, h->elem_grid, h->stream);
+    // device output needs no host-side total: the triangles follow at once, and the
+    // total arrives with them
+    if (on_device && max_tri > 0)
+        launch_surface_emit(G, n, h->P.nb, h->nbe, (uint32_t)env, scale, iso, (float)dx, h->surf, tri,
+                            (uint64_t)max_tri, h->stream);
     CK(cudaGetLastError());
-    uint32_t total = 0;
-    CK(cudaMemcpyAsync(&total, h->surf_counts + cells, sizeof total, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(h->h_total, h->surf.sums + sz.units, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    const uint32_t total = *h->h_total;
     *n_tri = total;
     const uint64_t nwrite = std::min<uint64_t>(total, (uint64_t)max_tri);
-    if (nwrite == 0) return MPM_OK;
-    float *dst = tri;
-    if (!on_device) {
-        size_t cap = h->surf_tri_cap;
-        if (cap < nwrite) {   // the old buffer stays with the handle until mpm_destroy
-            if ((st = ensure(h, &h->surf_tri, &cap, 9 * (size_t)nwrite)) != MPM_OK) return st;
-            h->surf_tri_cap = nwrite;
-        }
-        dst = h->surf_tri;
+    if (nwrite == 0 || on_device) return MPM_OK;
+    size_t cap = h->surf_tri_cap;
+    if (cap < nwrite) {   // the old buffer stays with the handle until mpm_destroy
+        if ((st = ensure(h, &h->surf_tri, &cap, 9 * (size_t)nwrite)) != MPM_OK) return st;
+        h->surf_tri_cap = nwrite;
     }
-    launch_surface_emit(G, n, h->P.nb, h->nbe, (uint32_t)env, scale, iso, (float)dx, h->surf_counts, dst, nwrite,
-                        h->elem_grid, h->stream);
+    float *dst = h->surf_tri;
+    launch_surface_emit(G, n, h->P.nb, h->nbe, (uint32_t)env, scale, iso, (float)dx, h->surf, dst, nwrite, h->stream);
     CK(cudaGetLastError());
-    if (!on_device)
-        CK(cudaMemcpyAsync(tri, dst, sizeof(float) * 9 * nwrite, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(tri, dst, sizeof(float) * 9 * nwrite, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return MPM_OK;
 }

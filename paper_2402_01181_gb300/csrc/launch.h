@@ -78,14 +78,23 @@ void launch_reverse_step(bool do_p2g, bool do_g2p, const DevParams &P, const Rev
                          cudaStream_t st, bool dependent);
 
 // kernels_surface.cu: iso-surface of the grid density m / (rho dx^3) of
-// environment env.  counts: (n-1)^3 + 1 entries, left holding the exclusive
-// prefix of the per-cell triangle counts (last entry: the total); sums:
-// ceil(((n-1)^3 + 1) / 1024) + 1 entries.
-void launch_surface_count_scan(const float4 *G, int n, int nb, uint32_t nbe, uint32_t env, float scale, float iso,
-                               uint32_t *counts, uint32_t *sums, int grid, cudaStream_t st);
+// environment env.
+struct SurfaceSizes {
+    size_t bits;     // words of inside bits, 32 nodes of a row each
+    size_t words;    // words of cells, 32 of a row each
+    size_t units;    // groups of 32 words of cells
+};
+SurfaceSizes surface_sizes(int n);
+struct SurfaceScratch {
+    uint32_t *bits;      // SurfaceSizes::bits
+    uint16_t *counts;    // SurfaceSizes::words: triangles
+    uint32_t *sums;      // SurfaceSizes::units + 1: exclusive prefix of the triangles, then their total
+};
+void launch_surface_count(const float4 *G, int n, int nb, uint32_t nbe, uint32_t env, float scale, float iso,
+                          const SurfaceScratch &S, int grid, cudaStream_t st);
 // triangles (9 floats each) in cell order, the first max_tri of them
 void launch_surface_emit(const float4 *G, int n, int nb, uint32_t nbe, uint32_t env, float scale, float iso, float dx,
-                         const uint32_t *offsets, float *tri, uint64_t max_tri, int grid, cudaStream_t st);
+                         const SurfaceScratch &S, float *tri, uint64_t max_tri, cudaStream_t st);
 
 // kernels_sort.cu: stable counting sort of particles by grid block at load.
 struct SortScratch {

@@ -1,5 +1,7 @@
 """Several sub-steps per launch, the configuration a load chooses, and the
-readout at the edges of its warps."""
+readout and surface kernels at the edges of their warps and words."""
+import ctypes as ct
+
 import numpy as np
 import pytest
 
@@ -112,3 +114,32 @@ def test_device_readout_of_any_subset(M, n):
             got = t[k].cpu().numpy()
             assert np.array_equal(got, ref) if k in want else np.all(got == -7.0), (want, k)
     sim.close()
+
+
+@pytest.mark.parametrize("grid", [8, 16, 32, 64])
+@pytest.mark.parametrize("iso", [-1.0, 0.05, 0.5, 1.5, 1e6])
+def test_surface_of_scattered_particles(M, grid, iso):
+    """Ragged surfaces on rows of less than one, one and two 32-cell words, all
+    inside and all outside, against the oracle on the same FP32 density.  With
+    exact inputs the two differences and the quotient of an edge point are each
+    correctly rounded (3 x 2^-24 of a cell), its sum and product to 2^-23 of the
+    unit cube: 4e-7 in all."""
+    rng = np.random.default_rng(grid)
+    n = 6 * grid * grid
+    x = ((0.6 + (grid - 2.2) * rng.random((n, 3))) / grid).astype(np.float32)     # every stencil in the grid
+    sc = scenes.Scene("dust", n_grid=grid, dt=1e-5, E=1e3, nu=0.3, rho=1e3, x=x,
+                      particle_volume=(1.0 / grid) ** 3 / 3, bound=1)
+    sim = M.sim_from_scene(sc)
+    field = sim.read_grid()[..., 0] * np.float32(1.0 / (sc.rho * sc.dx ** 3))
+    ref = O.surface(field.astype(np.float64), np.float32(iso), sc.dx)
+    got = sim.extract_surface(iso)
+    dev = sim.extract_surface(iso, device=True).cpu().numpy()
+    room = max(1, len(ref) // 2)
+    part = np.zeros((room, 3, 3), np.float32)
+    count = ct.c_int64()
+    M.check(M.mpm_extract_surface(sim.h, 0, iso, part.ctypes.data_as(ct.c_void_p), room, ct.byref(count), 0))
+    sim.close()
+    assert got.shape == ref.shape and count.value == len(ref)
+    assert np.array_equal(got, dev) and np.array_equal(part[:len(ref)], got[:room])
+    assert len(ref) == 0 or np.abs(got - ref).max() <= 4e-7
+    assert (len(ref) > 0) == (field.min() < iso <= field.max())
