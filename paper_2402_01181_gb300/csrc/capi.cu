@@ -310,6 +310,7 @@ void fill_frames(mpm_handle *h, int first, int nsub, int total, int tstride, Too
             }
             reach += std::max(0.0, (double)h->cfg.theta);
             reach = reach * 1.001 + 1e-6;
+            const CallMotion<double> motion = call_motion(tl.cur, tl.tgt);
             for (int k = 0; k < nsub; ++k) {
                 const double s = (double)(first + k + 1) / (double)total;
                 ToolFrame &f = out[((size_t)k * h->n_envs + e) * tstride + t];
@@ -317,7 +318,7 @@ void fill_frames(mpm_handle *h, int first, int nsub, int total, int tstride, Too
                 f.kind = tl.kind;
                 if (tl.kind == MPM_TOOL_NONE) continue;
                 double R[9], T[3], u[3], w[3];
-                call_frame(tl.cur, tl.tgt, s, span, R, T, u, w);
+                call_frame(motion, tl.cur, tl.tgt, s, span, R, T, u, w);
                 for (int i = 0; i < 9; ++i) f.R[i] = (float)R[i];
                 for (int a = 0; a < 3; ++a) {
                     f.T[a] = (float)T[a];
@@ -557,9 +558,8 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     if ((st = dalloc_t(h, &h->fb.vc.vc1, N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->fb.vc.vc2, N)) != MPM_OK) return bail(st);
     const int ngrid = cfg->pipeline == MPM_PIPELINE_FUSED ? 3 : 1;
-    for (int g = 0; g < ngrid; ++g)
-        if ((st = dalloc_t(h, &h->fb.G[g], nn)) != MPM_OK) return bail(st);
-    for (int g = ngrid; g < 3; ++g) h->fb.G[g] = h->fb.G[0];
+    if ((st = dalloc_t(h, &h->fb.G[0], ngrid * nn)) != MPM_OK) return bail(st);
+    for (int g = 1; g < 3; ++g) h->fb.G[g] = h->fb.G[0] + (g < ngrid ? g * nn : 0);
     if ((st = dalloc_t(h, &h->fb.ctrl, 1)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->staging, 24 * N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->d_frames, (size_t)h->sub_chunk * n_envs * MPM_MAX_TOOLS)) != MPM_OK) return bail(st);
@@ -595,6 +595,7 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     if (e != cudaSuccess) return bail(fail(MPM_ERR_ALLOC, "cudaMallocHost: %s", cudaGetErrorString(e)));
     *h->h_err = 0;
     h->h_total = h->h_err + 1;
+    h->fb.host_err = h->h_err;
     if ((e = cudaEventCreateWithFlags(&h->ev_err, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[0], cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[1], cudaEventDisableTiming)) != cudaSuccess ||
@@ -722,7 +723,7 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
     if (is_fused(h)) {
-        for (int g = 0; g < 3; ++g) CK(cudaMemsetAsync(h->fb.G[g], 0, sizeof(float4) * nn, h->stream));
+        CK(cudaMemsetAsync(h->fb.G[0], 0, 3 * sizeof(float4) * nn, h->stream));
         CK(cudaMemsetAsync(h->sort.counts, 0, sizeof(uint32_t) * h->nblocks, h->stream));
         launch_block_sort(h->P, dx, (uint32_t)n, h->sort, h->fb.ctrl, h->elem_grid, h->stream);
         const int par = cur_par(h);
@@ -867,7 +868,10 @@ mpm_status mpm_step(mpm_handle *h, int32_t n_substeps) {
     }
     h->taken += n_substeps;
     for (auto &t : h->tools) std::memcpy(t.cur, t.tgt, sizeof t.cur);
-    return enqueue_error_copy(h);
+    if (!is_fused(h)) return enqueue_error_copy(h);
+    CK(cudaEventRecord(h->ev_err, h->stream));     // the last launch left the error bits in h_err
+    h->err_pending = true;
+    return MPM_OK;
 }
 
 mpm_status mpm_synchronize(mpm_handle *h) {
@@ -920,7 +924,12 @@ mpm_status mpm_read_particles(mpm_handle *h, float *x, float *v, float *F, float
         }
         CK(cudaGetLastError());
     }
-    return mpm_synchronize(h);
+    if (!is_fused(h) || !h->err_pending) return mpm_synchronize(h);
+    // whatever sets error bits on the fused pipeline (loads, sub-steps) also sends
+    // them to h_err before it records ev_err
+    CK(cudaStreamSynchronize(h->stream));
+    CK(cudaEventSynchronize(h->ev_err));
+    return status_of(*h->h_err);
 }
 
 static mpm_status ensure_dense(mpm_handle *h) {

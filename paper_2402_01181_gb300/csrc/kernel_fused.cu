@@ -876,6 +876,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             __threadfence();
             if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
             ctrl->done = 0;
+            *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
             if (RECORD) *rec.nact = nact;
             ctrl->step = step + 1;
         }

@@ -132,23 +132,41 @@ void qmatrix(const QuatT<S> &q, S R[9]) {
     R[6] = 2.0 * (x * z - w * y); R[7] = 2.0 * (y * z + w * x); R[8] = 1.0 - 2.0 * (x * x + y * y);
 }
 
+// The rotation of a call from pose0 to pose1: where it starts and the rotation
+// vector it turns by, the same for all of the call's sub-steps.
+template <class S>
+struct CallMotion {
+    QuatT<S> q0;
+    S phi[3];
+};
+template <class S>
+CallMotion<S> call_motion(const S pose0[6], const S pose1[6]) {
+    CallMotion<S> m;
+    m.q0 = qexp_rotvec(pose0 + 3);
+    const QuatT<S> q1 = qexp_rotvec(pose1 + 3);
+    const QuatT<S> dq = qmul(q1, QuatT<S>{m.q0.w, -m.q0.x, -m.q0.y, -m.q0.z});
+    qlog_rotvec(dq, m.phi);
+    return m;
+}
+template <class S>
+void call_frame(const CallMotion<S> &m, const S pose0[6], const S pose1[6], double s, double span, S R[9], S T[3],
+                S u[3], S w[3]) {
+    const S rs[3] = {s * m.phi[0], s * m.phi[1], s * m.phi[2]};
+    qmatrix(qmul(qexp_rotvec(rs), m.q0), R);
+    for (int a = 0; a < 3; ++a) {
+        T[a] = pose0[a] + s * (pose1[a] - pose0[a]);
+        u[a] = (pose1[a] - pose0[a]) / span;
+        w[a] = m.phi[a] / span;
+    }
+}
+
 // The frame of a tool at fraction s in (0, 1] of a call that moves it
 // uniformly from pose0 to pose1 (T, rotation vector) in span seconds:
 // T(s) = T0 + s (T1 - T0), R(s) = exp(s phi) R0 with phi = log(R1 R0^T), and
 // the rigid velocity u = (T1 - T0) / span, w = phi / span.
 template <class S>
 void call_frame(const S pose0[6], const S pose1[6], double s, double span, S R[9], S T[3], S u[3], S w[3]) {
-    const QuatT<S> q0 = qexp_rotvec(pose0 + 3), q1 = qexp_rotvec(pose1 + 3);
-    const QuatT<S> dq = qmul(q1, QuatT<S>{q0.w, -q0.x, -q0.y, -q0.z});
-    S phi[3];
-    qlog_rotvec(dq, phi);
-    const S rs[3] = {s * phi[0], s * phi[1], s * phi[2]};
-    qmatrix(qmul(qexp_rotvec(rs), q0), R);
-    for (int a = 0; a < 3; ++a) {
-        T[a] = pose0[a] + s * (pose1[a] - pose0[a]);
-        u[a] = (pose1[a] - pose0[a]) / span;
-        w[a] = phi[a] / span;
-    }
+    call_frame(call_motion(pose0, pose1), pose0, pose1, s, span, R, T, u, w);
 }
 
 }  // namespace gbmpm
