@@ -68,7 +68,8 @@ struct FusedSmem {
     uint4 inbox[2][kInbox];
     EnvParams ep[2];               // the block's environment: material
     ToolFrame tools[2][kMaxTools]; // and its tool frames for this sub-step
-    uint32_t items[2], bids[2];
+    uint32_t items[2], bids[2];    // work items (their place in the lists) and their blocks (kNoBlock: none)
+    uint32_t own;                  // a block that this CTA keeps for the launch's next sub-step, or kNoBlock
     int acc[4][kArena];            // P2G arena over nodes [4b-1, 4b+6]^3 (fixed point, padded strides)
     // staged P2G inputs of one group: packed arena base, fx (3), q (3), A dx (9)
     int st_base[GROUP];
@@ -229,7 +230,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     using Smem = FusedSmem<T, GP, PD>;
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
     constexpr int NW = Smem::NW, GROUP = Smem::GROUP;
-    constexpr bool kEarly = T * MINB <= 512;
+    constexpr bool kEarly = T * MINB <= 512, kKeep = MINB == 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     Ctrl *ctrl = B.ctrl;
     const int par = step & 1, m3 = step % 3;
@@ -248,7 +249,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     const uint32_t nheavy = (uint32_t)nhl, nact = (uint32_t)nhl + (uint32_t)(nhl >> 32);
     const uint32_t acap = B.nblocks;
     auto item_block = [&](uint32_t it) -> uint32_t {
-        return it >= s.nact ? 0u : __ldcg(&B.alist[0][blk_in + (it < s.nheavy ? it : acap - 1u - (it - s.nheavy))]);
+        return it >= s.nact ? kNoBlock : __ldcg(&B.alist[0][blk_in + (it < s.nheavy ? it : acap - 1u - (it - s.nheavy))]);
     };
     const uint32_t nclr = *(volatile uint32_t *)&ctrl->nclear[(step + 3u) & 3u];     // G_{k-1}'s
     const uint32_t *__restrict__ clr = B.clist[m3c];
@@ -258,23 +259,42 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     const uint32_t nbe = P.nbe;
     uint32_t err = 0;
 
-    // prologue: this CTA's first work item and its inputs (the shared counter hands
-    // out items gridDim.x, gridDim.x + 1, ... afterwards).
-    // The first gridDim.x items are the front of the heavy list, then the light
+    // prologue: this CTA's first block and its inputs.  With one CTA per SM (kKeep)
+    // that is, after the launch's first sub-step, the block it kept, known without a
+    // memory access, so that its inputs are under way before the lists' sizes
+    // arrive; the lists then hold the blocks that no CTA kept (8K cube 444 -> 424 us a
+    // frame, 2K patch 109 -> 106; with two CTAs per SM a fixed placement loses more
+    // where two heavy blocks share an SM: the 30K slab's reset 408 -> 438).  Otherwise
+    // the first gridDim.x items are the front of the heavy list, then the light
     // list's, each CTA's at a place that does not depend on the lists' sizes: both
-    // entries are read together with the sizes.
-    if (tid == 0) { s.m3 = (uint32_t)m3; s.nact = nact; s.nheavy = nheavy; }
+    // entries are read together with the sizes.  The shared counter hands out the rest.
+    const bool lists = !kKeep || first;
+    const uint32_t fixed = lists ? gridDim.x : 0u;     // items that the counter starts from
     if (tid == T - 1) {
-        const uint32_t back = gridDim.x - 1u - blockIdx.x;     // this CTA's place in the light list
-        const uint32_t *al = B.alist[0] + blk_in;
-        const uint32_t hb = blockIdx.x < acap ? __ldcg(&al[blockIdx.x]) : 0u;
-        const uint32_t lb = back < acap ? __ldcg(&al[acap - 1u - back]) : 0u;
-        const bool heavy = blockIdx.x < nheavy;
-        s.items[0] = heavy ? blockIdx.x : nheavy + back;
-        s.bids[0] = heavy ? hb : lb;
+        uint32_t item = 0, b;
+        if (lists) {
+            const uint32_t back = gridDim.x - 1u - blockIdx.x;     // this CTA's place in the light list
+            const uint32_t *al = B.alist[0] + blk_in;
+            const uint32_t hb = blockIdx.x < acap ? __ldcg(&al[blockIdx.x]) : 0u;
+            const uint32_t lb = back < acap ? __ldcg(&al[acap - 1u - back]) : 0u;
+            const bool heavy = blockIdx.x < nheavy;
+            item = heavy ? blockIdx.x : nheavy + back;
+            b = item >= nact ? kNoBlock : heavy ? hb : lb;
+        } else {
+            b = s.own;
+            if (b == kNoBlock && nact > 0u) {
+                item = atomicAdd(&ctrl->work[m3], 1u);
+                if (item < nact)
+                    b = __ldcg(&B.alist[0][blk_in + (item < nheavy ? item : acap - 1u - (item - nheavy))]);
+            }
+        }
+        s.items[0] = item;
+        s.bids[0] = b;
+        s.own = kNoBlock;
     }
     __syncthreads();
-    if (s.items[0] < nact) prefetch_block<T>(s, 0, s.bids[0], B.inbox[0], blk_in, Gcur, P, tools, tid);
+    if (s.bids[0] != kNoBlock) prefetch_block<T>(s, 0, s.bids[0], B.inbox[0], blk_in, Gcur, P, tools, tid);
+    if (tid == 0) { s.m3 = (uint32_t)m3; s.nact = nact; s.nheavy = nheavy; }
     // the P2G arena starts at zero; every flush returns the nodes it read to zero
     if (first)
         for (int q = tid; q < 4 * kArena; q += T) (&s.acc[0][0])[q] = 0;
@@ -296,20 +316,19 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     __syncthreads();
 
     for (int cb = 0;; cb ^= 1) {
-        const uint32_t item = s.items[cb];
-        if (item >= s.nact) break;
         const uint32_t b = s.bids[cb];                 // global block
-        if (RECORD && tid == 0) rec.act[item] = b;
+        if (b == kNoBlock) break;
+        if (RECORD && tid == 0) rec.act[s.items[cb]] = b;
         const uint32_t env = b >> (3 * P.lnb);          // environment
         const uint32_t eb0 = env * nbe;                 // its first global block
         int bx, by, bz;
         block_coords(b, P.lnb, bx, by, bz);
         const EnvParams &ep = s.ep[cb];
         const float m = ep.mass;
-        // the next work item: the atomic is issued here and its result is
-        // consumed after this thread's share of the grid operation
-        uint32_t next_item = 0;
-        if (tid == T - 1) next_item = gridDim.x + atomicAdd(&ctrl->work[s.m3], 1u);
+        // the next work item, unless the lists hold none: the atomic is issued here and
+        // its result is consumed after this thread's share of the grid operation
+        uint32_t next_item = s.nact;
+        if (tid == T - 1 && s.nact > fixed) next_item = fixed + atomicAdd(&ctrl->work[s.m3], 1u);
         uint32_t alloc_ob = 0, alloc_cf = 0;     // thread 0: the block's output range and chunks
         float4 *gv = s.graw[cb];
 
@@ -439,7 +458,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 t.stamp = 0; t.first = 0; t.npass = 0;
             }
             B.tabs[0][blk_out + b] = t;
-            if (RECORD) rec.blk[item] = make_uint2(fit ? alloc_ob : 0u, fit ? total : 0u);
+            if (RECORD) rec.blk[s.items[cb]] = make_uint2(fit ? alloc_ob : 0u, fit ? total : 0u);
             s.out_base = fit ? alloc_ob : nparticles;
             s.chunk_first = fit ? alloc_cf : nchunk_cap;
         }
@@ -451,7 +470,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)(T + tid), tid, 1);
             cp_async_commit();
         }
-        if (s.items[cb ^ 1] < s.nact) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
+        if (s.bids[cb ^ 1] != kNoBlock) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
         else cp_async_commit();
         const int ox = 4 * bx - 1, oy = 4 * by - 1, oz = 4 * bz - 1;   // arena origin
 
@@ -475,10 +494,13 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             if (warp == NW - 2) {
                 B.clist[(step + 1u) % 3u][atomicAdd(&ctrl->nclear[(step + 1) & 3u], 1u)] = mark_b;
             } else {
-                // heavy: b itself (lane 13) with more particles now than one pass of the
-                // CTA takes.  A neighbour's mark wins only for blocks that particles
+                // kKeep: b itself (lane 13) stays with this CTA if it keeps no other; into
+                // the lists goes the rest.  Heavy: b with more particles now than one pass of
+                // the CTA takes.  A neighbour's mark wins only for blocks that particles
                 // enter from outside, which are light.
-                if (lane == 13 && total > (uint32_t)T)
+                if (kKeep && !last && lane == 13 && s.own == kNoBlock)
+                    s.own = mark_b;
+                else if (lane == 13 && total > (uint32_t)T)
                     B.alist[0][blk_out + atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][0], 1u)] = mark_b;
                 else
                     B.alist[0][blk_out + acap - 1u - atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][1], 1u)] = mark_b;
