@@ -231,6 +231,11 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
     constexpr int NW = Smem::NW, GROUP = Smem::GROUP;
     constexpr bool kEarly = T * MINB <= 512, kKeep = MINB == 1;
+    // Particles over which a block is heavy: one pass of the CTA.  With two CTAs per SM
+    // a scene has about a block per CTA, and half a pass tells a full block of a sparse
+    // slab from one at its edge: CTA i and the one a wave later, which share an SM,
+    // then take one of each (30K slab 368 -> 340 us a frame in contact).
+    constexpr uint32_t kHeavy = MINB == 2 ? T / 2 : T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     Ctrl *ctrl = B.ctrl;
     const int par = step & 1, m3 = step % 3;
@@ -495,12 +500,12 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 B.clist[(step + 1u) % 3u][atomicAdd(&ctrl->nclear[(step + 1) & 3u], 1u)] = mark_b;
             } else {
                 // kKeep: b itself (lane 13) stays with this CTA if it keeps no other; into
-                // the lists goes the rest.  Heavy: b with more particles now than one pass of
-                // the CTA takes.  A neighbour's mark wins only for blocks that particles
+                // the lists goes the rest.  Heavy: b with more than kHeavy particles now.  A
+                // neighbour's mark wins only for blocks that particles
                 // enter from outside, which are light.
                 if (kKeep && !last && lane == 13 && s.own == kNoBlock)
                     s.own = mark_b;
-                else if (lane == 13 && total > (uint32_t)T)
+                else if (lane == 13 && total > kHeavy)
                     B.alist[0][blk_out + atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][0], 1u)] = mark_b;
                 else
                     B.alist[0][blk_out + acap - 1u - atomicAdd(&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][1], 1u)] = mark_b;

@@ -228,7 +228,9 @@ __global__ void __launch_bounds__(256) k_init_tables(DevParams P, const uint32_t
             B.tabs[par][b] = t;
             B.inbox[par][(size_t)b * kInbox + 13 * kNpMax] = make_uint4(off, c, step, 0u);
             B.astamp[b] = step;
-            B.alist[par][atomicAdd(&B.ctrl->nactive[m3][0], 1u)] = b;
+            // the sub-step kernel's lists: heavy blocks from the front, light from the back
+            if (c > 128u) B.alist[par][atomicAdd(&B.ctrl->nactive[m3][0], 1u)] = b;
+            else B.alist[par][m - 1u - atomicAdd(&B.ctrl->nactive[m3][1], 1u)] = b;
         }
         if (lane >= 27) continue;
         B.chunks[par][b].run[lane] = make_uint2(lane == 13 ? off : 0u, lane == 13 ? c : 0u);
