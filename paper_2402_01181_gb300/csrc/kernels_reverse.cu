@@ -40,7 +40,7 @@ constexpr int kRevThreads = 128;
 // their second round spares the two tiles' round trip (gradients of a 100-sub-step
 // rollout, 30K particles: 128 5.17, 256 5.02, 512 5.02 ms).
 constexpr uint32_t kChunk = 256, kMaxChunks = 16;
-// Lanes per particle: 1 (the whole stencil; a chunk is then one round of the
+// Lanes per particle: 1 (the whole stencil; a chunk is then two rounds of the
 // CTA) or 3 (one z-plane of the stencil each, partials summed by shuffles),
 // which made the whole backward 4% slower.
 constexpr int kRevLanes = 1;
