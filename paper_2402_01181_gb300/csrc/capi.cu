@@ -147,7 +147,7 @@ struct mpm_handle {
     ToolFrame *h_frames[2] = {nullptr, nullptr};
     int frames_next = 0;
     uint32_t *h_err = nullptr;       // pinned copy of Ctrl::err
-    uint32_t *h_total = nullptr;     // pinned: number of triangles of a surface
+    uint32_t *h_total = nullptr;     // pinned scratch word: triangles of a surface, error bits
     cudaEvent_t ev_err = nullptr, ev_frames[2] = {nullptr, nullptr};
     // the reverse pass's segment replays run on their own stream, one segment
     // ahead of the reverse sub-steps: rp_rec[b] marks record buffer b complete,
@@ -886,8 +886,11 @@ mpm_status mpm_synchronize(mpm_handle *h) {
 mpm_status mpm_clear_error(mpm_handle *h) {
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
+    CK(cudaMemcpyAsync(h->h_total, &h->fb.ctrl->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemsetAsync(&h->fb.ctrl->err, 0, sizeof(uint32_t), h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    // a launch whose CTAs lost one another left its counters anywhere: load again
+    if (*h->h_total & kErrStall) h->loaded = false;
     *h->h_err = 0;
     h->err_pending = false;
     return MPM_OK;
