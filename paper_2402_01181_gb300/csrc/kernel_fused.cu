@@ -918,7 +918,8 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&ctrl->done) : "memory");
         } while (now < target && ++polls < kMaxPolls);
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        if (now < target) atomicOr(&ctrl->err, kErrStall);
+        if (now < target)      // nobody reaches the end of the launch, where the host's copy is written
+            *(volatile uint32_t *)B.host_err = atomicOr(&ctrl->err, kErrStall) | kErrStall;
         s.go = now >= target;
     }
     __syncthreads();
