@@ -638,6 +638,15 @@ namespace {
 
 mpm_status apply_kernel_config(mpm_handle *h, int config);
 
+// The loaded particles' volume in full 4x4x4 blocks.
+double full_blocks(const mpm_handle *h) {
+    const double cell = 1.0 / ((double)h->P.n * h->P.n * h->P.n);
+    double full = 0.0;
+    for (int e = 0; e < h->n_envs; ++e)
+        full += (double)(h->env_off[e + 1] - h->env_off[e]) * h->env_vol[e] / (64.0 * cell);
+    return full;
+}
+
 static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuration follows the selectable ones");
 // The fused sub-step's configuration for the loaded particles, where the caller
 // has set none.  By the number of filled 4x4x4 blocks, estimated as the particles
@@ -653,10 +662,7 @@ static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuratio
 //   run from 4 to 5 blocks per CTA on with the most warps (500K at 8 per cell 51.4,
 //   59, 61, 50.5, 70; 800K 72.4, 81, 86, 76.3, 106; 1M 94, 105, 109, 100, 138).
 int choose_config(const mpm_handle *h) {
-    const double cell = 1.0 / ((double)h->P.n * h->P.n * h->P.n), sms = h->num_sms;
-    double full = 0.0;
-    for (int e = 0; e < h->n_envs; ++e)
-        full += (double)(h->env_off[e + 1] - h->env_off[e]) * h->env_vol[e] / (64.0 * cell);
+    const double sms = h->num_sms, full = full_blocks(h);
     const bool sparse = (double)h->n < 6.0 * 64.0 * full;
     const double blocks = full * (sparse ? 2.0 : 1.5);
     if (blocks <= sms) return kConfigT512;
@@ -720,6 +726,10 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     if (is_fused(h) && !h->config_set) {
         const int config = choose_config(h);
         if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
+        // a few CTAs for every block (a body may spread), not one per SM: each more
+        // arrives at and polls the wait between sub-steps (2K patch 104 -> 100 us a call)
+        if (config == kConfigT512)
+            h->fused_grid = std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
     }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
     if (is_fused(h)) {

@@ -46,7 +46,9 @@ def test_calls_of_several_lengths_follow_the_oracle(M, config):
 
 
 @pytest.mark.parametrize("n,ppc,grid,threads,ctas_per_sm", [
-    (8192, 16.0, 32, 512, 1),        # 8 blocks' worth: a block's chain, the fewest passes
+    (1, 16.0, 32, 512, -32),         # at least 32 CTAs
+    (8192, 16.0, 32, 512, -48),      # 8 blocks' worth: a block's chain, the fewest passes, 6 CTAs a block
+    (45000, 9.0, 64, 512, 1),        # 78: one CTA per SM at most
     (30000, 3.18, 64, 256, 2),       # 147: a CTA for every block, no spills
     (800000, 9.0, 128, 256, 3),      # 1389, dense
     (50000, 3.2, 64, 128, 4),        # 244, sparse
@@ -60,7 +62,7 @@ def test_load_chooses_by_size_and_density(M, n, ppc, grid, threads, ctas_per_sm)
     sim = M.Sim(cfg)
     sim.load(x, 1.0 / (ppc * grid ** 3))
     got = sim.kernel_config()
-    assert got == {"config": 0, "threads": threads, "ctas": ctas_per_sm * sms}
+    assert got == {"config": 0, "threads": threads, "ctas": -ctas_per_sm if ctas_per_sm < 0 else ctas_per_sm * sms}
     sim.set_kernel_config(2)         # a set one is kept by later loads
     sim.load(x, 1.0 / (ppc * grid ** 3))
     assert sim.kernel_config()["config"] == 2 and sim.kernel_config()["threads"] == 128
