@@ -20,12 +20,12 @@
 //   4. P2G (Eqs. 1-3) of up to 2 passes of new particle states at a time into an
 //      8^3-node shared arena around b.  The arena accumulates in 32-bit fixed
 //      point with native shared integer atomics (shared float atomics are
-//      several times slower): mass in units of m_p 2^-22, momentum in units of
-//      B 2^-22 where B bounds every contribution of the group, so no
-//      contribution exceeds 2^22 and no node sum of <= 512 particles can
-//      overflow; the integer sums are exact, hence independent of the order of
-//      the atomics.  A particle that moved further than one cell scatters
-//      straight into G_{k+1} with float atomics instead.
+//      several times slower): mass in units of m_p 2^-23, momentum in units of
+//      B 2^-23 where B bounds every value that the group scatters (2^-22 in
+//      groups of 1,024).  Weights are at most 0.42, so no contribution exceeds
+//      2^22 and no node sum can overflow; the integer sums are exact, hence
+//      independent of the order of the atomics.  A particle that moved further
+//      than one cell scatters straight into G_{k+1} with float atomics instead.
 //   5. the arena is converted back to floats and added to G_{k+1} with float4
 //      atomics (only the 6^3 nodes around b when every base cell lies in b),
 //      and the nodes read are returned to zero.
@@ -47,7 +47,11 @@ namespace {
 
 constexpr uint32_t kMaxPolls = 1u << 22;   // of the wait between sub-steps: a few seconds
 constexpr int CMAX = 512;      // run candidates (source chunk x direction) per block
-constexpr float kFix = 4194304.0f;      // 2^22
+// Fixed-point units per bound of a group of up to 512 or 1,024 particles: 2^23 or
+// 2^22.  A weight is at most 0.75^3 = 0.42, so a term stays below 2^22 (kMagic's
+// range) and a node's sum of all the group's terms below 2^31.
+template <int GROUP>
+constexpr float kFixUnits = GROUP <= 512 ? 8388608.0f : 4194304.0f;
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: float -> nearest int for |v| < 2^22
 // arena node (x, y, z) in [0,8)^3 sits at x + kAy y + kAz z: kAz = 68 keeps the
 // bases of a z-pair of cells in distinct shared-memory banks
@@ -230,6 +234,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     using Smem = FusedSmem<T, GP, PD>;
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
     constexpr int NW = Smem::NW, GROUP = Smem::GROUP;
+    constexpr float kFix = kFixUnits<GROUP>;
     constexpr bool kEarly = T * MINB <= 512, kKeep = MINB == 1;
     // Particles over which a block is heavy: one pass of the CTA.  With two CTAs per SM
     // a scene has about a block per CTA, and half a pass tells a full block of a sparse
@@ -644,10 +649,11 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                     s.st_q[0][slot] = qx; s.st_q[1][slot] = qy; s.st_q[2][slot] = qz;
 #pragma unroll
                     for (int q = 0; q < 9; ++q) s.st_a[q][slot] = A[q];
-                    // bound of |q + A' o| over the stencil, per component
-                    const float b0 = fabsf(qx) + 2.f * (fabsf(A[0]) + fabsf(A[1]) + fabsf(A[2]));
-                    const float b1 = fabsf(qy) + 2.f * (fabsf(A[3]) + fabsf(A[4]) + fabsf(A[5]));
-                    const float b2 = fabsf(qz) + 2.f * (fabsf(A[6]) + fabsf(A[7]) + fabsf(A[8]));
+                    // bound of |q + A' o| over the stencil, per component: about its centre
+                    // o = (1, 1, 1)
+                    const float b0 = fabsf(qx + (A[0] + A[1] + A[2])) + (fabsf(A[0]) + fabsf(A[1]) + fabsf(A[2]));
+                    const float b1 = fabsf(qy + (A[3] + A[4] + A[5])) + (fabsf(A[3]) + fabsf(A[4]) + fabsf(A[5]));
+                    const float b2 = fabsf(qz + (A[6] + A[7] + A[8])) + (fabsf(A[6]) + fabsf(A[7]) + fabsf(A[8]));
                     const float bp = fmaxf(fmaxf(b0, b1), b2);
                     bound = isfinite(bp) ? __float_as_uint(bp) : 0u;
                 } else {
@@ -812,7 +818,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                     // momentum inputs in fixed-point units, as (x, y) and (z, mass)
                     // pairs for the packed f32x2 pipe: the value at stencil offset
                     // (ii, jj, kk) is q + A' (ii, jj, kk), the mass term the constant
-                    // kFix (m_p 2^22 in mass units)
+                    // kFix (m_p in mass units)
                     const float2 sv2 = make_float2(sv, sv), two = make_float2(2.f, 2.f);
                     const float2 qxy = __fmul2_rn(make_float2(s.st_q[0][q], s.st_q[1][q]), sv2);
                     const float2 qzm = make_float2(s.st_q[2][q] * sv, kFix);
