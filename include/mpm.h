@@ -303,7 +303,9 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
  * mpm_set_tool_pose with those poses and mpm_step(1) n_substeps times.
  * The handle's state advances to the end of the rollout.  The particle state
  * is stored every checkpoint_every sub-steps (24 floats per particle each);
- * mpm_tape_backward recomputes the sub-steps in between.  The paper does not
+ * mpm_tape_backward recomputes the sub-steps in between, unless
+ * MPM_PIPELINE_FUSED keeps the record of them all, which it does up to 8 GiB
+ * and a sixteenth of the device's free memory.  The paper does not
  * differentiate its simulator (Sec. V names differentiable physics as future
  * work); this is the plain reverse mode of the sub-step defined above.
  * Needs a handle with one environment (MPM_ERR_STATE otherwise), on either

@@ -104,7 +104,10 @@ struct Tape {
     float4 *lp = nullptr;             // 2 x 3 n: state adjoints by position within a segment
     size_t cap_lp = 0;
     bool last_recorded = false;       // the record buffers hold the last segment (from the forward pass)
-    int nbuf = 1;                     // record buffers: 2 when there is more than one segment
+    // record buffers: one per segment where they fit (kept_record), so that nothing
+    // is replayed; otherwise 2 when there is more than one segment
+    int nbuf = 1;
+    uint32_t end_step = 0;            // h->step at the rollout's end
 };
 
 }  // namespace
@@ -1122,6 +1125,22 @@ size_t rs_floats(int64_t n) { return 24 * (size_t)n + 2 * (((size_t)n + 3) & ~si
 // work list (1 per block) and the list length (padded to 4 words)
 size_t rs_words(const mpm_handle *h) { return 3 * (size_t)h->nblocks + 4; }
 
+// Whether the record of a whole rollout of nck segments of ck sub-steps is kept:
+// up to 8 GiB, and a sixteenth of what the device has free, unless the handle has
+// that much from an earlier rollout.  The replays that it spares cost about as much
+// as the forward pass and share the SMs with the reverse sub-steps (30K particles,
+// 100 sub-steps, gradients: 4.95 -> 4.41 ms, a segment recorded in one launch).
+bool keeps_record(const mpm_handle *h, int64_t n, int ck, int nck) {
+    const Tape &tp = h->tape;
+    const size_t nn = (size_t)h->P.n * h->P.n * h->P.n, steps = (size_t)ck * nck;
+    const size_t floats = rs_floats(n) * steps, grids = 2 * nn * steps, words = rs_words(h) * steps;
+    if (tp.cap_rs >= floats && tp.cap_rsg >= grids && tp.cap_rsb >= words) return true;
+    const size_t bytes = sizeof(float) * floats + sizeof(float4) * grids + sizeof(uint32_t) * words;
+    size_t free_b = 0, total_b = 0;
+    if (bytes > (size_t)8 << 30 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+    return bytes <= free_b / 16;
+}
+
 // Sub-step j of record buffer buf (segment sg is recorded in buffer sg % nbuf).
 StepRecord step_record(mpm_handle *h, int j, int buf) {
     Tape &tp = h->tape;
@@ -1144,13 +1163,17 @@ StepRecord step_record(mpm_handle *h, int j, int buf) {
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n;
     r.grid = tp.rs_grid + 2 * slot * nn;
     r.vgrid = r.grid + nn;
+    r.floats = rs_floats(tp.n);
+    r.words = rs_words(h);
+    r.nodes = 2 * nn;
     return r;
 }
 
-// The fused state as an image by particle id: x (3n), v (3n), F (9n), C (9n).
-void id_image(mpm_handle *h, float *img) {
+// The fused state as an image by particle id: x (3n), v (3n), F (9n), C (9n); vc:
+// its v and C, by position.
+void id_image(mpm_handle *h, const VCState &vc, float *img) {
     const size_t n = (size_t)h->n;
-    launch_read_out(cur_state(h), h->fb.vc, (uint32_t)n, img, img + 3 * n, img + 6 * n, img + 15 * n, h->elem_grid,
+    launch_read_out(cur_state(h), vc, (uint32_t)n, img, img + 3 * n, img + 6 * n, img + 15 * n, h->elem_grid,
                     h->stream);
 }
 
@@ -1191,7 +1214,7 @@ mpm_status replay_segment(mpm_handle *h, int sg, cudaStream_t r) {
     if (st == MPM_OK) {
         for (int j = 0; j < len; ++j) {
             launch_fused_step_record(h->P, h->fb, tp.frames + (size_t)(c0 + j) * tp.ntools, step_record(h, j, b),
-                                     record_grid(h), r);
+                                     1, record_grid(h), r);
             h->step += 1u;
         }
     }
@@ -1235,9 +1258,10 @@ mpm_status fused_reverse(mpm_handle *h, const AdjState &A, int nck) {
     // the reverse grid operation: one wave of 3 CTAs per SM (a node per thread
     // over 8 list entries per work-list block, most of them empty)
     const int adj_grid_ctas = 3 * h->num_sms;
+    const bool have_all = tp.nbuf == nck;     // every segment's record comes from the forward pass
     const bool have_last = tp.last_recorded;
-    tp.last_recorded = false;     // the replays below overwrite the record buffers
-    const bool ahead = tp.nbuf == 2;
+    tp.last_recorded = false;     // replays overwrite the record buffers
+    const bool ahead = tp.nbuf == 2 && !have_all;
     cudaStream_t r = s;
     if (ahead) {
         if ((st = ensure_replay_stream(h)) != MPM_OK) return st;
@@ -1254,7 +1278,7 @@ mpm_status fused_reverse(mpm_handle *h, const AdjState &A, int nck) {
     }
     for (int sg = nck - 1; sg >= 0; --sg) {
         const int c0 = sg * tp.ck, len = std::min(tp.ck, tp.nsub - c0), b = sg % tp.nbuf;
-        const bool replayed = !(sg == nck - 1 && have_last);
+        const bool replayed = !have_all && !(sg == nck - 1 && have_last);
         if (replayed) {
             if (ahead) {
                 CK(cudaStreamWaitEvent(s, h->rp_rec[b], 0));
@@ -1319,6 +1343,8 @@ mpm_status fused_reverse(mpm_handle *h, const AdjState &A, int nck) {
     R.lame_part = tp.lame_part;
     launch_reverse_step(true, false, h->P, R, h->rev_grid, s, true);
     CK(cudaGetLastError());
+    // without replays, and with nothing stepped or loaded since, the live state is still the rollout's end
+    if (have_all && h->step == tp.end_step) return enqueue_error_copy(h);
     return load_image(h, tp.final_img);
 }
 
@@ -1357,19 +1383,29 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
         tp.image = 24 * (size_t)n;
         if ((st = ensure(h, &tp.ckpt, &tp.cap_ckpt, tp.image * nck)) != MPM_OK) return st;
         if ((st = ensure(h, &tp.final_img, &tp.cap_final, tp.image)) != MPM_OK) return st;
-        // two record buffers when there are several segments: the reverse pass
-        // replays a segment into one while it reverses the one in the other
-        const int nbuf = nck > 1 ? 2 : 1;
-        if ((st = ensure(h, &tp.rs, &tp.cap_rs, rs_floats(n) * ck * nbuf)) != MPM_OK) return st;
-        if (tp.cap_rsg < 2 * nn * ck * nbuf) {
-            // recorded sub-steps write the grid (before and after the grid operation)
-            // over their blocks' regions only; the reverse grid operation also reads the
-            // rest of the blocks it lists, where it needs finite values (its adjoint
-            // there is zero)
-            if ((st = ensure(h, &tp.rs_grid, &tp.cap_rsg, 2 * nn * ck * nbuf)) != MPM_OK) return st;
-            CK(cudaMemsetAsync(tp.rs_grid, 0, sizeof(float4) * 2 * nn * ck * nbuf, h->stream));
+        // a record buffer for every segment where that is little memory; otherwise two
+        // when there are several: the reverse pass replays a segment into one while
+        // it reverses the one in the other
+        int nbuf = keeps_record(h, n, ck, nck) ? nck : std::min(nck, 2);
+        auto reserve = [&](size_t steps) -> mpm_status {
+            mpm_status r = ensure(h, &tp.rs, &tp.cap_rs, rs_floats(n) * steps);
+            if (r == MPM_OK && tp.cap_rsg < 2 * nn * steps) {
+                // recorded sub-steps write the grid (before and after the grid operation)
+                // over their blocks' regions only; the reverse grid operation also reads the
+                // rest of the blocks it lists, where it needs finite values (its adjoint
+                // there is zero)
+                if ((r = ensure(h, &tp.rs_grid, &tp.cap_rsg, 2 * nn * steps)) != MPM_OK) return r;
+                CK(cudaMemsetAsync(tp.rs_grid, 0, sizeof(float4) * 2 * nn * steps, h->stream));
+            }
+            return r != MPM_OK ? r : ensure(h, &tp.rs_blk, &tp.cap_rsb, rs_words(h) * steps);
+        };
+        st = reserve((size_t)ck * nbuf);
+        if (st == MPM_ERR_ALLOC && nbuf > 2) {
+            cudaGetLastError();
+            nbuf = 2;
+            st = reserve((size_t)ck * nbuf);
         }
-        if ((st = ensure(h, &tp.rs_blk, &tp.cap_rsb, rs_words(h) * ck * nbuf)) != MPM_OK) return st;
+        if (st != MPM_OK) return st;
         tp.nbuf = nbuf;
         if ((st = ensure(h, &tp.gbar, &tp.cap_gb, nn)) != MPM_OK) return st;
         size_t one = tp.cap_gb;
@@ -1416,12 +1452,17 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
         tp.n = n;
         tp.ck = ck;
         const int c_last = (nck - 1) * ck, b_last = (nck - 1) % tp.nbuf;
+        const bool all = tp.nbuf == nck;
         for (int k = 0; k < n_substeps;) {
-            if (k % ck == 0) id_image(h, tp.ckpt + (size_t)(k / ck) * tp.image);
+            // a recording sub-step leaves v and C in its record
+            const bool recorded = k > 0 && (all || k > c_last);
+            const VCState before = recorded ? step_record(h, (k - 1) % ck, (k - 1) / ck % tp.nbuf).vc : h->fb.vc;
+            if (k % ck == 0) id_image(h, before, tp.ckpt + (size_t)(k / ck) * tp.image);
             int m = 1;
-            if (k >= c_last) {
-                launch_fused_step_record(h->P, h->fb, tp.frames + (size_t)k * nt, step_record(h, k - c_last, b_last),
-                                         record_grid(h), h->stream);
+            if (all || k >= c_last) {
+                m = std::min(ck, n_substeps - k);
+                launch_fused_step_record(h->P, h->fb, tp.frames + (size_t)k * nt, step_record(h, 0, k / ck % tp.nbuf),
+                                         m, record_grid(h), h->stream);
             } else {
                 // the configuration the reverse pass replays segments with, so that the
                 // replay follows the recorded trajectory up to the order of float atomics
@@ -1438,8 +1479,9 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
         CK(cudaMemcpyAsync(h->fb.vc.vc0, rv.vc0, 16 * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
         CK(cudaMemcpyAsync(h->fb.vc.vc1, rv.vc1, 16 * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
         CK(cudaMemcpyAsync(h->fb.vc.vc2, rv.vc2, 16 * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
-        id_image(h, tp.final_img);
+        id_image(h, h->fb.vc, tp.final_img);
         tp.last_recorded = true;
+        tp.end_step = h->step;
     } else {
         for (int k = 0; k < n_substeps; ++k) {
             if (k % ck == 0 && (st = live_to_image(h, tp.ckpt + (size_t)(k / ck) * tp.image)) != MPM_OK) return st;

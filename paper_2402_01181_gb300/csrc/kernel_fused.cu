@@ -100,6 +100,7 @@ struct FusedSmem {
     uint32_t ncand, total, out_base, chunk_first, npass, mask, bmax, wide;
     uint32_t nact, nheavy;         // active blocks, heavy ones among them
     uint32_t m3;                   // sub-step index mod 3
+    StepRecord rec;                // the sub-step's record (recording sub-steps)
     bool go;                       // the launch's next sub-step may start
 };
 
@@ -112,6 +113,16 @@ static_assert(4 * (sizeof(FusedSmem<128, 2>) + 1024) <= 228 * 1024, "shared memo
 static_assert(5 * (sizeof(FusedSmem<128, 1>) + 1024) <= 228 * 1024, "shared memory for five CTAs per SM");
 static_assert(4 * (sizeof(FusedSmem<128, 2, 2>) + 1024) <= 228 * 1024, "configuration 2: four CTAs per SM");
 static_assert(2 * (sizeof(FusedSmem<256, 2, 2>) + 1024) <= 228 * 1024, "configuration 4: two CTAs per SM");
+
+// the record k sub-steps after r
+__host__ __device__ __forceinline__ StepRecord record_of(StepRecord r, uint32_t k) {
+    const size_t f = k * r.floats, w = k * r.words, g = k * r.nodes;
+    r.xi += f / 4; r.f0 += f / 4; r.f1 += f / 4; r.f2 += f; r.src += f;
+    r.vc.vc0 += f / 4; r.vc.vc1 += f / 4; r.vc.vc2 += f / 4;
+    r.blk += w / 2; r.act += w; r.nact += w;
+    r.grid += g; r.vgrid += g;
+    return r;
+}
 
 __device__ __forceinline__ BlockTab load_tab(const BlockTab *p) {
     const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
@@ -229,7 +240,7 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 // after the last sub-step, or when the wait for the other CTAs ran out.
 template <bool WRITE_VC, int T, int GP, int MINB, bool RECORD, int PD>
 __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const DevParams &P, const FusedBufs &B,
-                                              const ToolFrame *__restrict__ tools, const StepRecord &rec,
+                                              const ToolFrame *__restrict__ tools, const StepRecord &rec0, uint32_t k,
                                               uint32_t step, uint32_t target, bool first, bool last) {
     using Smem = FusedSmem<T, GP, PD>;
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
@@ -280,6 +291,8 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     // entries are read together with the sizes.  The shared counter hands out the rest.
     const bool lists = !kKeep || first;
     const uint32_t fixed = lists ? gridDim.x : 0u;     // items that the counter starts from
+    const StepRecord &rec = s.rec;
+    if (RECORD && tid == 0) s.rec = record_of(rec0, k);
     if (tid == T - 1) {
         uint32_t item = 0, b;
         if (lists) {
@@ -321,6 +334,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
         ctrl->nactive[m3c][0] = 0;
         ctrl->nactive[m3c][1] = 0;
         ctrl->nclear[(step + 2u) & 3u] = 0;
+        if (RECORD) *rec.nact = nact;
     }
     cp_async_wait_all();
     __syncthreads();
@@ -910,7 +924,6 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
             ctrl->done = 0;
             *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
-            if (RECORD) *rec.nact = nact;
             ctrl->step = step + 1;
         }
         return false;
@@ -952,11 +965,11 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FusedSmem<T, GP, PD> &s = *reinterpret_cast<FusedSmem<T, GP, PD> *>(smem_raw);
     const uint32_t step = *(volatile uint32_t *)&B.ctrl->step;
-    if constexpr (!kManySteps<T, MINB> || RECORD) {
-        fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools, rec, step, gridDim.x, true, true);
+    if constexpr (!kManySteps<T, MINB>) {
+        fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
     } else {
         for (uint32_t k = 0;; ++k)
-            if (!fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools + (size_t)k * frames, rec, step + k,
+            if (!fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools + (size_t)k * frames, rec, k, step + k,
                                                                   (k + 1) * gridDim.x, k == 0, k + 1 == nsub))
                 break;
     }
@@ -984,7 +997,7 @@ void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, c
         cudaGetLastError();
         cfg.numAttrs = 0;
         for (int k = 0; k < nsub; ++k)
-            cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, rec, 1u);
+            cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, record_of(rec, k), 1u);
     }
 }
 
@@ -1045,8 +1058,9 @@ int fused_record_occupancy() {
 }
 
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
-                              int grid, cudaStream_t st) {
-    launch_steps(k_fused_step<false, 256, 2, 2, true>, 256, sizeof(FusedSmem<256, 2>), P, B, tools, rec, 1, grid, st);
+                              int nsub, int grid, cudaStream_t st) {
+    launch_steps(k_fused_step<false, 256, 2, 2, true>, 256, sizeof(FusedSmem<256, 2>), P, B, tools, rec, nsub, grid,
+                 st);
 }
 
 // Also opts the kernel into its dynamic shared memory size on the current

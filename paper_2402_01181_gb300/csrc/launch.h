@@ -155,6 +155,9 @@ struct StepRecord {
     float4 *grid;        // the grid the sub-step read, over the 6^3 region of every listed block (node layout)
     float4 *vgrid;       // the grid velocities after the grid operation (.xyz), over the same regions
     VCState vc;          // each particle's v and C after the sub-step (n entries, same order as xi)
+    // from one sub-step's record to the next one's: floats of the particle arrays,
+    // words of blk, act and nact, nodes of the grids
+    size_t floats, words, nodes;
 };
 // Inputs and outputs of one reverse sub-step (kernels_reverse.cu).
 struct ReverseArgs {
@@ -196,8 +199,9 @@ int fused_step_occupancy(int config);
 bool fused_many_steps(int config);     // whether a launch takes many sub-steps
 int fused_step_threads(int config);
 int fused_record_occupancy();
+// nsub recording sub-steps, rec the first one's record.
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
-                              int grid, cudaStream_t st);
+                              int nsub, int grid, cudaStream_t st);
 constexpr int kConfigT512 = 5;          // beside the MPM_KERNEL_CONFIGS that a caller can select
 constexpr int kFusedMinThreads = 128;     // chunk tables are sized for the smallest CTA
 // Inbox of a block: entry d * kNpMax + p holds the run of source pass p

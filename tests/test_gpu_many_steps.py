@@ -145,3 +145,54 @@ def test_surface_of_scattered_particles(M, grid, iso):
     assert np.array_equal(got, dev) and np.array_equal(part[:len(ref)], got[:room])
     assert len(ref) == 0 or np.abs(got - ref).max() <= 4e-7
     assert (len(ref) > 0) == (field.min() < iso <= field.max())
+
+
+def _lattice_sim(M, grid, lo, hi):
+    sc = scenes.Scene("lattice", n_grid=grid, dt=2e-5, E=5e3, nu=0.3, rho=1e3,
+                      x=scenes.jittered_lattice((lo,) * 3, (hi,) * 3, grid, (2, 2, 2), seed=3),
+                      particle_volume=(1.0 / grid) ** 3 / 8)
+    return M.sim_from_scene(H.perturbed_scene(sc, seed=4, v_scale=0.05, c_scale=0.5, f_dev=0.02))
+
+
+def _agree(a, b):
+    """The bounds of the segmented backward: 1e-4 of the largest entry."""
+    for k in ("E", "nu"):
+        assert abs(a[k] - b[k]) <= 1e-4 * abs(a[k]), k
+    for k in ("x", "v", "F", "C"):
+        ga, gb = a[k].cpu().numpy(), b[k].cpu().numpy()
+        assert np.abs(ga - gb).max() <= 1e-4 * np.abs(ga).max(), k
+
+
+def test_rollout_too_large_to_keep_is_replayed(M):
+    """140 sub-steps on a 128^3 grid take 9.4 GB of record, over the 8 GiB that are
+    kept: four segments, replayed through two buffers, against one segment,
+    which the forward pass records whatever its size."""
+    import torch
+    out = []
+    for ck in (140, 35):
+        sim = _lattice_sim(M, 128, 60, 66)
+        sim.tape_record(np.zeros((140, 0, 6)), ck)
+        g = torch.Generator(device="cuda").manual_seed(5)
+        xbar = 1e-4 * torch.randn((sim.n, 3), generator=g, device="cuda")
+        out.append(sim.tape_backward(xbar, want_state=True))
+        sim.close()
+    _agree(*out)
+
+
+def test_kept_record_serves_a_second_backward_and_the_state_is_the_rollouts_end(M):
+    import torch
+    sim = _lattice_sim(M, 32, 12, 18)
+    sim.tape_record(np.zeros((11, 0, 6)), 4)
+    end = sim.read()
+    g = torch.Generator(device="cuda").manual_seed(6)
+    bars = [1e-3 * torch.randn((sim.n, c), generator=g, device="cuda") for c in (3, 3, 9, 9)]
+    first = sim.tape_backward(*bars, want_state=True)
+    assert all(np.array_equal(sim.read()[k], end[k]) for k in end)
+    sim.step(2)                                  # the record does not depend on the live state
+    _agree(first, sim.tape_backward(*bars, want_state=True))
+    assert all(np.array_equal(sim.read()[k], end[k]) for k in end)
+    one = _lattice_sim(M, 32, 12, 18)
+    one.tape_record(np.zeros((11, 0, 6)), 11)
+    _agree(one.tape_backward(*bars, want_state=True), first)
+    one.close()
+    sim.close()
