@@ -90,6 +90,13 @@ def kernel_source_sha():
     return h.hexdigest()[:16]
 
 
+def config_name(sim, best):
+    from paper_2402_01181_gb300 import mpm
+    if sim.kernel_config()["threads"] == 512:
+        return "512 threads, 2 passes per flush (the load's own choice)"
+    return mpm.KERNEL_CONFIG_NAMES[best]
+
+
 def fused_launches(sim, substeps, device):
     """Launches of the fused kernel per call of `substeps` sub-steps: one per
     sub-step at 80 registers a thread (768 threads per SM), one for all and one
@@ -270,7 +277,7 @@ def run_gpu_workload(name, args, rank, device, barrier, max_over_ranks, with_e2e
                   "ms_per_step_by_config": None}
     elif pipe == mpm.MPM_PIPELINE_FUSED and not args.no_autotune:
         best, times = sim.autotune(S)          # restores the state it starts from
-        tuning = {"config": best, "name": mpm.KERNEL_CONFIG_NAMES[best], "ms_per_step_by_config": times}
+        tuning = {"config": best, "name": config_name(sim, best), "ms_per_step_by_config": times}
 
     def frame():
         s = s_next[0]
@@ -361,7 +368,7 @@ def run_batched(args, rank, device, barrier, max_over_ranks, steps=6, loop_steps
     tuning = None
     if not args.no_autotune:
         best, times = sim.autotune(S)
-        tuning = {"config": best, "name": mpm.KERNEL_CONFIG_NAMES[best], "ms_per_step_by_config": times}
+        tuning = {"config": best, "name": config_name(sim, best), "ms_per_step_by_config": times}
     s_next = [0]
 
     def set_tools():
