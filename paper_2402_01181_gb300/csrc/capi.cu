@@ -1106,15 +1106,10 @@ mpm_status copy_in(float *dst, const float *src, size_t count, int on_device, cu
     return MPM_OK;
 }
 
-// The fused-kernel configuration of a recorded rollout (its forward pass and
-// the segment replays of its reverse pass): 256 threads, 2 passes per flush,
-// 2 CTAs per SM.
-constexpr int kRecordConfig = 4;
+// CTAs of a recorded rollout's sub-steps (its forward pass and the segment replays
+// of its reverse pass).
 int record_grid(mpm_handle *h) {
-    if (h->rec_grid == 0) {
-        fused_step_occupancy(kRecordConfig);    // opts the configuration into its shared memory
-        h->rec_grid = h->num_sms * std::max(fused_record_occupancy(), 1);
-    }
+    if (h->rec_grid == 0) h->rec_grid = h->num_sms * std::max(fused_rollout_occupancy(), 1);
     return h->rec_grid;
 }
 
@@ -1464,11 +1459,8 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
                 launch_fused_step_record(h->P, h->fb, tp.frames + (size_t)k * nt, step_record(h, 0, k / ck % tp.nbuf),
                                          m, record_grid(h), h->stream);
             } else {
-                // the configuration the reverse pass replays segments with, so that the
-                // replay follows the recorded trajectory up to the order of float atomics
                 m = std::min(ck, n_substeps - k);
-                launch_fused_steps(h->P, h->fb, tp.frames + (size_t)k * nt, m, true, record_grid(h), kRecordConfig,
-                                   h->stream);
+                launch_fused_steps_rollout(h->P, h->fb, tp.frames + (size_t)k * nt, m, record_grid(h), h->stream);
             }
             h->step += (uint32_t)m;
             k += m;

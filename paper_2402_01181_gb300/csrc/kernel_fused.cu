@@ -22,7 +22,7 @@
 //      point with native shared integer atomics (shared float atomics are
 //      several times slower): mass in units of m_p 2^-23, momentum in units of
 //      B 2^-23 where B bounds every value that the group scatters (2^-22 in
-//      groups of 1,024).  Weights are at most 0.42, so no contribution exceeds
+//      groups of 1,024 and in recorded rollouts).  Weights are at most 0.42, so no contribution exceeds
 //      2^22 and no node sum can overflow; the integer sums are exact, hence
 //      independent of the order of the atomics.  A particle that moved further
 //      than one cell scatters straight into G_{k+1} with float atomics instead.
@@ -47,11 +47,19 @@ namespace {
 
 constexpr uint32_t kMaxPolls = 1u << 22;   // of the wait between sub-steps: a few seconds
 constexpr int CMAX = 512;      // run candidates (source chunk x direction) per block
+// What a launch belongs to: plain stepping, or a recorded rollout (mpm_tape_record),
+// whose sub-steps keep their records (kRecord) or not (kRollout).
+enum Use { kStep, kRollout, kRecord };
 // Fixed-point units per bound of a group of up to 512 or 1,024 particles: 2^23 or
 // 2^22.  A weight is at most 0.75^3 = 0.42, so a term stays below 2^22 (kMagic's
-// range) and a node's sum of all the group's terms below 2^31.
-template <int GROUP>
-constexpr float kFixUnits = GROUP <= 512 ? 8388608.0f : 4194304.0f;
+// range) and a node's sum of all the group's terms below 2^31.  Rollouts keep 2^22
+// and the bound about the stencil's base: the pose gradients of a rollout in contact
+// hang on which nodes under the tool stick and which slide, and a rounding that
+// every run shares moves them by more than one run differs from another (30K slab,
+// 100 sub-steps: by 1.0e-4 of their norm with 2^23 and the bound about the centre,
+// runs differ by 2.4e-5).
+template <int GROUP, Use USE>
+constexpr float kFixUnits = GROUP <= 512 && USE == kStep ? 8388608.0f : 4194304.0f;
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: float -> nearest int for |v| < 2^22
 // arena node (x, y, z) in [0,8)^3 sits at x + kAy y + kAz z: kAz = 68 keeps the
 // bases of a z-pair of cells in distinct shared-memory banks
@@ -239,7 +247,7 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 
 
 // MINB: resident CTAs per SM the configuration is compiled for (the register budget)
-// RECORD: also write, for the reverse mode, every block's input particles at
+// USE kRecord: also write, for the reverse mode, every block's input particles at
 // their output positions (inside the range [out_base, out_base + total) the
 // block's output was allocated) with their input positions, the list of
 // blocks in work order with each one's range, the list's length, and the grid
@@ -248,14 +256,15 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 // launch's last (WRITE_VC: the one that writes v and C).  target: CTAs of the
 // launch times its sub-steps up to this one.  Returns whether to go on: false
 // after the last sub-step, or when the wait for the other CTAs ran out.
-template <bool WRITE_VC, int T, int GP, int MINB, bool RECORD, int PD>
+template <bool WRITE_VC, int T, int GP, int MINB, Use USE, int PD>
 __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const DevParams &P, const FusedBufs &B,
                                               const ToolFrame *__restrict__ tools, const StepRecord &rec0, uint32_t k,
                                               uint32_t step, uint32_t target, bool first, bool last) {
     using Smem = FusedSmem<T, GP, PD>;
     static_assert(PD == 1 || PD == 2, "one or two particle copies in flight");
     constexpr int NW = Smem::NW, GROUP = Smem::GROUP;
-    constexpr float kFix = kFixUnits<GROUP>;
+    constexpr bool RECORD = USE == kRecord;
+    constexpr float kFix = kFixUnits<GROUP, USE>;
     constexpr bool kEarly = T * MINB <= 512, kKeep = MINB == 1;
     // Particles over which a block is heavy: one pass of the CTA.  With two CTAs per SM
     // a scene has about a block per CTA, and half a pass tells a full block of a sparse
@@ -687,10 +696,14 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                     s.st4[Smem::st(slot, 2)] = make_float4(A[0], A[3], A[1], A[4]);
                     s.st4[Smem::st(slot, 3)] = make_float4(A[2], A[5], A[7], A[8]);
                     // bound of |q + A' o| over the stencil, per component: about its centre
-                    // o = (1, 1, 1)
-                    const float b0 = fabsf(qx + (A[0] + A[1] + A[2])) + (fabsf(A[0]) + fabsf(A[1]) + fabsf(A[2]));
-                    const float b1 = fabsf(qy + (A[3] + A[4] + A[5])) + (fabsf(A[3]) + fabsf(A[4]) + fabsf(A[5]));
-                    const float b2 = fabsf(qz + (A[6] + A[7] + A[8])) + (fabsf(A[6]) + fabsf(A[7]) + fabsf(A[8]));
+                    // o = (1, 1, 1), or its base
+                    auto bound_of = [](float q, float ai, float aj, float ak) {
+                        const float r = fabsf(ai) + fabsf(aj) + fabsf(ak);
+                        return USE == kStep ? fabsf(q + (ai + aj + ak)) + r : fabsf(q) + 2.f * r;
+                    };
+                    const float b0 = bound_of(qx, A[0], A[1], A[2]);
+                    const float b1 = bound_of(qy, A[3], A[4], A[5]);
+                    const float b2 = bound_of(qz, A[6], A[7], A[8]);
                     const float bp = fmaxf(fmaxf(b0, b1), b2);
                     bound = isfinite(bp) ? __float_as_uint(bp) : 0u;
                 } else {
@@ -982,7 +995,7 @@ constexpr bool kManySteps = T * MINB <= 640;
 // before.  One launch for all of them spares the launch gap and the ramp of the
 // CTAs between sub-steps; the CTAs then wait for one another, so nsub > 1 needs
 // a cooperative launch.  v and C are written by the last one (if WRITE_VC).
-template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, bool RECORD = false, int PD = 1>
+template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, Use USE = kStep, int PD = 1>
 __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B,
                                                         const ToolFrame *__restrict__ tools, uint32_t frames,
                                                         StepRecord rec, uint32_t nsub) {
@@ -990,10 +1003,10 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     FusedSmem<T, GP, PD> &s = *reinterpret_cast<FusedSmem<T, GP, PD> *>(smem_raw);
     const uint32_t step = *(volatile uint32_t *)&B.ctrl->step;
     if constexpr (!kManySteps<T, MINB>) {
-        fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
+        fused_substep<WRITE_VC, T, GP, MINB, USE, PD>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
     } else {
         for (uint32_t k = 0;; ++k)
-            if (!fused_substep<WRITE_VC, T, GP, MINB, RECORD, PD>(s, P, B, tools + (size_t)k * frames, rec, k, step + k,
+            if (!fused_substep<WRITE_VC, T, GP, MINB, USE, PD>(s, P, B, tools + (size_t)k * frames, rec, k, step + k,
                                                                   (k + 1) * gridDim.x, k == 0, k + 1 == nsub))
                 break;
     }
@@ -1036,20 +1049,20 @@ void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *too
     const int plain = !write_vc ? nsub : kOne ? 0 : nsub - 1;
     const int per = kManySteps<T, MINB> ? plain : 1;
     for (int k = 0; k < plain; k += per)
-        launch_steps(k_fused_step<false, T, GP, MINB, false, PD>, T, smem, P, B, tools + k * frames, none, per, grid, st);
+        launch_steps(k_fused_step<false, T, GP, MINB, kStep, PD>, T, smem, P, B, tools + k * frames, none, per, grid, st);
     if (plain < nsub)
-        launch_steps(k_fused_step<true, T, GP, MINB, false, PD>, T, smem, P, B, tools + plain * frames, none,
+        launch_steps(k_fused_step<true, T, GP, MINB, kStep, PD>, T, smem, P, B, tools + plain * frames, none,
                      nsub - plain, grid, st);
 }
 
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
 int variant_occupancy() {
     const int bytes = (int)sizeof(FusedSmem<T, GP, PD>);
-    cudaFuncSetAttribute(k_fused_step<true, T, GP, MINB, false, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    cudaFuncSetAttribute(k_fused_step<false, T, GP, MINB, false, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaFuncSetAttribute(k_fused_step<true, T, GP, MINB, kStep, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaFuncSetAttribute(k_fused_step<false, T, GP, MINB, kStep, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_fused_step<true, T, GP, MINB, false, PD>, T, bytes);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused_step<false, T, GP, MINB, false, PD>, T, bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_fused_step<true, T, GP, MINB, kStep, PD>, T, bytes);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused_step<false, T, GP, MINB, kStep, PD>, T, bytes);
     return a < b ? a : b;
 }
 
@@ -1071,20 +1084,28 @@ bool fused_many_steps(int config) { return config != 0 && config != 1; }
 
 int fused_step_threads(int config) { return config == 5 ? 512 : config == 2 || config == 3 ? 128 : 256; }
 
-// The recording sub-step of the differentiable rollout: the configuration of
-// 256 threads, 2 passes per flush and 2 CTAs per SM (128 registers).
-int fused_record_occupancy() {
-    constexpr int bytes = (int)sizeof(FusedSmem<256, 2>);
-    cudaFuncSetAttribute(k_fused_step<false, 256, 2, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    int a = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_fused_step<false, 256, 2, 2, true>, 256, bytes);
-    return a;
+// The sub-steps of a recorded rollout: 256 threads, 2 passes per flush and 2
+// CTAs per SM (128 registers); the recording ones copy particles one pass ahead.
+int fused_rollout_occupancy() {
+    constexpr int rec = (int)sizeof(FusedSmem<256, 2>), fwd = (int)sizeof(FusedSmem<256, 2, 2>);
+    cudaFuncSetAttribute(k_fused_step<false, 256, 2, 2, kRecord>, cudaFuncAttributeMaxDynamicSharedMemorySize, rec);
+    cudaFuncSetAttribute(k_fused_step<true, 256, 2, 2, kRollout, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd);
+    int a = 0, b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_fused_step<false, 256, 2, 2, kRecord>, 256, rec);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused_step<true, 256, 2, 2, kRollout, 2>, 256, fwd);
+    return a < b ? a : b;
 }
 
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
                               int nsub, int grid, cudaStream_t st) {
-    launch_steps(k_fused_step<false, 256, 2, 2, true>, 256, sizeof(FusedSmem<256, 2>), P, B, tools, rec, nsub, grid,
+    launch_steps(k_fused_step<false, 256, 2, 2, kRecord>, 256, sizeof(FusedSmem<256, 2>), P, B, tools, rec, nsub, grid,
                  st);
+}
+
+void launch_fused_steps_rollout(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, int grid,
+                                cudaStream_t st) {
+    launch_steps(k_fused_step<true, 256, 2, 2, kRollout, 2>, 256, sizeof(FusedSmem<256, 2, 2>), P, B, tools,
+                 StepRecord{}, nsub, grid, st);
 }
 
 // Also opts the kernel into its dynamic shared memory size on the current

@@ -198,10 +198,16 @@ void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame 
 int fused_step_occupancy(int config);
 bool fused_many_steps(int config);     // whether a launch takes many sub-steps
 int fused_step_threads(int config);
-int fused_record_occupancy();
-// nsub recording sub-steps, rec the first one's record.
+// Sub-steps of a recorded rollout: the CTAs per SM of both kinds (also opts them into
+// their dynamic shared memory), nsub recording ones, rec the first one's record, and
+// nsub ones without records, the last of which writes v and C.  Both kinds round
+// alike, so that a segment's replay follows the forward pass up to the order of
+// float atomics.
+int fused_rollout_occupancy();
 void launch_fused_step_record(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, const StepRecord &rec,
                               int nsub, int grid, cudaStream_t st);
+void launch_fused_steps_rollout(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, int grid,
+                                cudaStream_t st);
 constexpr int kConfigT512 = 5;          // beside the MPM_KERNEL_CONFIGS that a caller can select
 constexpr int kFusedMinThreads = 128;     // chunk tables are sized for the smallest CTA
 // Inbox of a block: entry d * kNpMax + p holds the run of source pass p
