@@ -948,20 +948,24 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     }
 
     if (err) atomicOr(&ctrl->err, err);
-    __syncthreads();
+    const bool failed = __syncthreads_or(err != 0u);
     // Arrivals count up over the launch's sub-steps, target = CTAs x sub-steps so
-    // far.  At the end of the launch's last one no fence: the last CTA reads only
-    // part_alloc, whose atomics every CTA consumed (its block's output range)
-    // before it arrived, and what it writes is read by the next launch.
-    // Elsewhere the arrival releases this CTA's writes and the wait acquires the
-    // others'.
+    // far.  At the end of the launch's last one the last CTA reads part_alloc, whose
+    // atomics every CTA consumed (its block's output range) before it arrived, and
+    // the error bits, so that a CTA that set some releases them with a fence before
+    // its arrival (the others need none); what the last CTA writes is read by the
+    // next launch.  Elsewhere the arrival releases this CTA's writes and the wait
+    // acquires the others'.
     if (last) {
-        if (tid == 0 && atomicAdd(&ctrl->done, 1u) == target - 1u) {
-            __threadfence();
-            if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
-            ctrl->done = 0;
-            *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
-            ctrl->step = step + 1;
+        if (tid == 0) {
+            if (failed) __threadfence();
+            if (atomicAdd(&ctrl->done, 1u) == target - 1u) {
+                __threadfence();
+                if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
+                ctrl->done = 0;
+                *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
+                ctrl->step = step + 1;
+            }
         }
         return false;
     }
