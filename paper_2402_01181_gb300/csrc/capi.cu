@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <string>
@@ -67,6 +68,7 @@ struct HostField {
 // vc1, vc2 (4 n floats each) then f2 (n floats, padded to a multiple of 4).
 struct Tape {
     bool valid = false;
+    bool settled = false;             // its launches are known to have run to their end
     int nsub = 0, ck = 0, ntools = 0;
     int64_t n = 0;
     size_t image = 0;                 // floats per state image
@@ -394,6 +396,17 @@ mpm_status poll_error(mpm_handle *h, bool wait) {
     return status_of(*h->h_err);
 }
 
+// A rollout whose recording launches lost one another has records of sub-steps that
+// never ran: it must not be reversed.  Waits for the launches, once per rollout.
+mpm_status settle_tape(mpm_handle *h) {
+    Tape &tp = h->tape;
+    if (!tp.valid || tp.settled) return MPM_OK;
+    CK(cudaEventSynchronize(h->ev_err));
+    tp.settled = true;
+    if (*h->h_err & kErrStall) tp.valid = false;
+    return MPM_OK;
+}
+
 mpm_status enqueue_error_copy(mpm_handle *h) {
     CK(cudaMemcpyAsync(h->h_err, &h->fb.ctrl->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaEventRecord(h->ev_err, h->stream));
@@ -498,6 +511,12 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     h->alloc_ctx = ctx;
     const char *ng = getenv("GBMPM_NO_GRAPHS");
     h->use_graphs = !(ng && ng[0] == '1');
+    // looks of the wait between two sub-steps of a launch: a few seconds' worth, or
+    // fewer by GBMPM_WAIT_POLLS (which lets a test make the wait run out)
+    h->fb.max_polls = 1u << 22;
+    const char *wp = getenv("GBMPM_WAIT_POLLS");
+    const long polls = wp ? std::strtol(wp, nullptr, 10) : 0;
+    if (polls > 0) h->fb.max_polls = (uint32_t)std::min<long>(polls, h->fb.max_polls);
 
     auto bail = [&](mpm_status st) {
         release_all(h);
@@ -798,6 +817,7 @@ mpm_status mpm_load_particles(mpm_handle *h, int64_t n, const float *x, const fl
     if (st != MPM_OK) return st;
     if (h->n_envs != 1) return fail(MPM_ERR_STATE, "a handle with several environments loads with mpm_load_batch");
     if (n < 0 || n > h->cfg.max_particles) return fail(MPM_ERR_ARG, "n = %lld outside [0, max_particles]", (long long)n);
+    if ((st = settle_tape(h)) != MPM_OK) return st;      // the load resets the error bits
     return load_impl(h, &n, x, v, F, C, &particle_volume, on_device);
 }
 
@@ -806,6 +826,7 @@ mpm_status mpm_load_batch(mpm_handle *h, const int64_t *counts, const float *x, 
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
     if (!counts || !particle_volumes) return fail(MPM_ERR_ARG, "NULL counts or particle volumes");
+    if ((st = settle_tape(h)) != MPM_OK) return st;
     return load_impl(h, counts, x, v, F, C, particle_volumes, on_device);
 }
 
@@ -899,6 +920,7 @@ mpm_status mpm_synchronize(mpm_handle *h) {
 mpm_status mpm_clear_error(mpm_handle *h) {
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
+    if ((st = settle_tape(h)) != MPM_OK) return st;
     CK(cudaMemcpyAsync(h->h_total, &h->fb.ctrl->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemsetAsync(&h->fb.ctrl->err, 0, sizeof(uint32_t), h->stream));
     CK(cudaStreamSynchronize(h->stream));
@@ -1489,6 +1511,7 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
     tp.ntools = nt;
     tp.n = n;
     tp.valid = true;
+    tp.settled = !tp.fused;
     return enqueue_error_copy(h);
 }
 
@@ -1501,7 +1524,8 @@ mpm_status mpm_tape_backward(mpm_handle *h, const float *x_bar, const float *v_b
     if (!tp.valid || tp.n != h->n) return fail(MPM_ERR_STATE, "no recorded rollout (mpm_tape_record) for this state");
     if (tool_stride(h) != tp.ntools || h->env_E[0] != tp.E || h->env_nu[0] != tp.nu)
         return fail(MPM_ERR_STATE, "tools or material changed since mpm_tape_record");
-    if ((st = poll_error(h, false)) != MPM_OK) return st;
+    if ((st = settle_tape(h)) != MPM_OK) return st;
+    if ((st = poll_error(h, !tp.valid)) != MPM_OK) return st;
     const int64_t n = tp.n;
     const int nt = tp.ntools;
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n;

@@ -45,7 +45,6 @@ namespace gbmpm {
 
 namespace {
 
-constexpr uint32_t kMaxPolls = 1u << 22;   // of the wait between sub-steps: a few seconds
 constexpr int CMAX = 512;      // run candidates (source chunk x direction) per block
 // What a launch belongs to: plain stepping, or a recorded rollout (mpm_tape_record),
 // whose sub-steps keep their records (kRecord) or not (kRollout).
@@ -971,12 +970,14 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
     }
     if (tid == 0) {
         // every CTA is resident (cooperative launch), so the wait ends when the last
-        // one arrives; after some seconds it ends with an error
+        // one arrives; after max_polls looks it ends with an error.  A CTA whose own
+        // look comes after the last arrival still goes on: every arrival was made, so it
+        // finds the sub-step before complete, and leaves at the next wait.
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctrl->done) : "memory");
         uint32_t now, polls = 0;
         do {
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&ctrl->done) : "memory");
-        } while (now < target && ++polls < kMaxPolls);
+        } while (now < target && ++polls < B.max_polls);
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
         if (now < target)      // nobody reaches the end of the launch, where the host's copy is written
             *(volatile uint32_t *)B.host_err = atomicOr(&ctrl->err, kErrStall) | kErrStall;
@@ -1006,6 +1007,11 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FusedSmem<T, GP, PD> &s = *reinterpret_cast<FusedSmem<T, GP, PD> *>(smem_raw);
     const uint32_t step = *(volatile uint32_t *)&B.ctrl->step;
+    // Behind a wait that ran out, the arrivals, counters and lists are those of a launch
+    // that its CTAs left at different sub-steps: nothing runs on them before the next
+    // load sets them anew.  (That keeps the lists in bounds: a block is appended once
+    // per stamp, to a counter that was zero.)
+    if (*(volatile uint32_t *)&B.ctrl->err & kErrStall) return;
     if constexpr (!kManySteps<T, MINB>) {
         fused_substep<WRITE_VC, T, GP, MINB, USE, PD>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
     } else {

@@ -133,6 +133,7 @@ struct FusedBufs {
     uint32_t *gstamp;         // per block: last sub-step it was put on a clear list
     Ctrl *ctrl;
     uint32_t *host_err;       // pinned host word that receives Ctrl::err at the end of a launch
+    uint32_t max_polls;       // of the wait between two sub-steps of a launch
     uint32_t nblocks;
     // the second buffer of P, chunks, tabs, alist and inbox follows the first in
     // one allocation: pstride slots, cstride chunks, nblocks blocks further on
