@@ -85,6 +85,8 @@ struct Tape {
     std::vector<double> pose_init;    // ntools x 6
     std::vector<double> poses;        // nsub x ntools x 6
     double E = 0, nu = 0;
+    EnvParams mat{};                  // the material and tool count it was recorded with
+    EnvParams *d_mat = nullptr;       // and their device copy, where the handle's have changed since
     // fused pipeline: checkpoints are particle-id-ordered images (x, v, F, C:
     // 24 floats per particle); the segment being reversed is replayed with
     // recording sub-steps, each keeping its input particles by block and the
@@ -1246,8 +1248,8 @@ mpm_status replay_segment(mpm_handle *h, int sg, cudaStream_t r) {
 // the first sub-step's P2G.  The record of a segment is made by replaying it
 // from its checkpoint; with two record buffers the replays run on their own
 // stream one segment ahead, beside the reverse of the segment after.  The
-// last segment's record comes from the forward pass.  The live state is
-// restored to the rollout's end.
+// last segment's record comes from the forward pass.  Replays leave their own
+// state in place of the live one.
 mpm_status fused_reverse(mpm_handle *h, const AdjState &A, int nck) {
     Tape &tp = h->tape;
     const int nt = tp.ntools;
@@ -1360,9 +1362,7 @@ mpm_status fused_reverse(mpm_handle *h, const AdjState &A, int nck) {
     R.lame_part = tp.lame_part;
     launch_reverse_step(true, false, h->P, R, h->rev_grid, s, true);
     CK(cudaGetLastError());
-    // without replays, and with nothing stepped or loaded since, the live state is still the rollout's end
-    if (have_all && h->step == tp.end_step) return enqueue_error_copy(h);
-    return load_image(h, tp.final_img);
+    return MPM_OK;
 }
 
 mpm_status copy_out(float *dst, const float *src, size_t count, int on_device, cudaStream_t st) {
@@ -1461,6 +1461,7 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
     if (nt > 0) CK(cudaMemcpy(tp.frames, hf.data(), sizeof(ToolFrame) * hf.size(), cudaMemcpyHostToDevice));
     tp.E = h->env_E[0];
     tp.nu = h->env_nu[0];
+    tp.mat = h->envp_host[0];
     if (tp.fused) {
         // checkpoints by particle id; v and C of a checkpointed state are written by
         // the sub-step before it.  The last segment runs with recording sub-steps,
@@ -1526,6 +1527,21 @@ mpm_status mpm_tape_backward(mpm_handle *h, const float *x_bar, const float *v_b
         return fail(MPM_ERR_STATE, "tools or material changed since mpm_tape_record");
     if ((st = settle_tape(h)) != MPM_OK) return st;
     if ((st = poll_error(h, !tp.valid)) != MPM_OK) return st;
+    // The rollout is reversed, and replayed, with the material it was recorded with:
+    // what the handle's table holds now may have been set or loaded since, and the
+    // tool stride may be another's.
+    if ((st = upload_env_params(h)) != MPM_OK) return st;
+    struct Material {
+        DevParams &P;
+        const EnvParams *live;
+        ~Material() { P.envp = live; }
+    } material{h->P, h->P.envp};
+    const bool same_material = std::memcmp(&tp.mat, &h->envp_host[0], sizeof tp.mat) == 0;
+    if (!same_material) {
+        if (!tp.d_mat && (st = dalloc_t(h, &tp.d_mat, 1)) != MPM_OK) return st;
+        CK(cudaMemcpyAsync(tp.d_mat, &tp.mat, sizeof tp.mat, cudaMemcpyHostToDevice, h->stream));
+        h->P.envp = tp.d_mat;
+    }
     const int64_t n = tp.n;
     const int nt = tp.ntools;
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n;
@@ -1543,7 +1559,13 @@ mpm_status mpm_tape_backward(mpm_handle *h, const float *x_bar, const float *v_b
     CK(cudaMemsetAsync(tp.red, 0, sizeof(double) * nred, s));
     const int nck = (tp.nsub + tp.ck - 1) / tp.ck;
     if (tp.fused) {
+        const bool replayed = tp.nbuf != nck;
         if ((st = fused_reverse(h, A, nck)) != MPM_OK) return st;
+        h->P.envp = material.live;
+        // the live state back to the rollout's end, which it still is without replays and
+        // with nothing stepped, loaded or set since
+        if ((replayed || h->step != tp.end_step || !same_material) && (st = load_image(h, tp.final_img)) != MPM_OK)
+            return st;
     }
     for (int sg = tp.fused ? -1 : nck - 1; sg >= 0; --sg) {
         const int c0 = sg * tp.ck, len = std::min(tp.ck, tp.nsub - c0);

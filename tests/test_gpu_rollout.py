@@ -1,4 +1,5 @@
-"""The recorded rollout: its pose gradients against recorded values."""
+"""The recorded rollout: its pose gradients against recorded values, and a
+handle that moves on between a record and its backward."""
 import json
 import os
 
@@ -47,3 +48,58 @@ def test_pose_gradients_are_the_recorded_ones(M):
     ref = np.array(gold["poses"])
     off = np.linalg.norm(np.mean(runs, axis=0) - ref) / np.linalg.norm(ref)
     assert off <= 2 * gold["spread"], off
+
+
+def _press(M, pipeline):
+    """The cube in slow motion under a capsule that has just reached it: scene, poses."""
+    sc = scenes.cube8k(3)
+    sc.v, sc.C, sc.F = scenes.random_state(sc.x, 4, v_scale=0.05, c_scale=0.5, f_dev=0.02)
+    cap = scenes.capsule_shape(0.06, 0.08)
+    p0, vel = np.array([0.47, 0.759, 0.51, 0.1, 0.1, 0.2]), np.array([0.2, -0.5, 0.1, 1.0, -1.0, 0.5])
+    sc.tools = [scenes.Tool(cap, lambda s: p0 + vel * sc.dt * (s + 1))]
+    pl = M.MPM_PIPELINE_FUSED if pipeline == "fused" else M.MPM_PIPELINE_SPLIT
+    return sc, M.sim_from_scene(sc, pipeline=pl, load=False), np.stack([sc.tools[0].pose(k) for k in range(12)])[:, None]
+
+
+@pytest.mark.parametrize("pipeline", ["fused", "split"])
+@pytest.mark.parametrize("between", ["E", "rho", "volume", "tool"])
+def test_backward_takes_the_material_of_the_record(M, pipeline, between):
+    """What is set, stepped or loaded between a record and its backward (and in
+    E's and the tool's case set back) leaves the gradients those of the recorded
+    rollout: to 1e-4 of the largest entry, the pose gradients to 1e-3 (they
+    hang on stick and slide)."""
+    import torch
+    sc, sim, poses = _press(M, pipeline)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    bars = [1e-3 * torch.randn((sc.n, c), generator=g, device="cuda") for c in (3, 3, 9, 9)]
+    far = np.array([0.1, 0.9, 0.1, 0.0, 0.0, 0.0])
+    out = []
+    for change in (False, True):
+        sim.load(sc.x, sc.particle_volume, sc.v, sc.F, sc.C)
+        sim.set_tool(0, far, [M.MPM_TOOL_NONE] + [0.0] * 7)
+        sim.set_tool(0, sc.tools[0].pose(-1), sc.tools[0].shape)
+        sim.tape_record(poses, 5)
+        end = sim.read()
+        if change and between == "E":
+            sim.set_env_material(0, 3 * sc.E, 0.2, sc.rho)
+            sim.step(1)
+            sim.set_env_material(0, sc.E, sc.nu, sc.rho)
+        elif change and between == "rho":
+            sim.set_env_material(0, sc.E, sc.nu, 2 * sc.rho)
+        elif change and between == "volume":
+            sim.load(sc.x, 2 * sc.particle_volume, sc.v, sc.F, sc.C)
+        elif change:
+            sim.set_tool(1, np.array([0.5, 0.5, 0.5, 0.0, 0.0, 0.0]), scenes.box_shape(0.02, 0.02, 0.02))
+            sim.step(1)
+            sim.set_tool(1, far, [M.MPM_TOOL_NONE] + [0.0] * 7)
+        out.append(sim.tape_backward(*bars, want_state=True))
+        if pipeline == "fused":
+            assert all(np.array_equal(sim.read()[k], end[k]) for k in end)
+    sim.close()
+    a, b = out
+    for k in ("E", "nu"):
+        assert abs(a[k] - b[k]) <= 1e-4 * abs(a[k]), (k, a[k], b[k])
+    for k in ("x", "v", "F", "C"):
+        assert (a[k] - b[k]).abs().max() <= 1e-4 * a[k].abs().max(), k
+    assert np.abs(a["poses"]).max() > 0
+    assert np.abs(a["poses"] - b["poses"]).max() <= 1e-3 * np.abs(a["poses"]).max()
