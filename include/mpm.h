@@ -172,7 +172,10 @@ mpm_status mpm_add_sampled_field(mpm_handle *h, int32_t res, const double origin
  * Asynchronous on the handle's stream.  The fused pipeline folds a stable
  * counting sort of the particles by 4x4x4-cell grid block into each sub-step;
  * a block may receive particles from at most 512 source chunks of 256
- * particles per sub-step (MPM_ERR_CAPACITY otherwise). */
+ * particles per sub-step (MPM_ERR_CAPACITY otherwise), or 1,024 of 128: where
+ * 128-thread CTAs step an environment of more than 62,080 particles, the
+ * handle allocates 8 KB per CTA for that at the load (refused, a load's own
+ * choice takes 256 threads). */
 mpm_status mpm_step(mpm_handle *h, int32_t n_substeps);
 
 /* mpm_read_particles without the wait, for streaming positions out while

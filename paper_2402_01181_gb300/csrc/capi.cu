@@ -137,6 +137,7 @@ struct mpm_handle {
     int tstride = 0;            // tool frames per environment in the uploaded table
     uint32_t nbe = 0;           // blocks per environment
     uint32_t nblocks = 0, chunk_cap = 0;   // over all environments
+    size_t runs_cap = 0;        // entries of fb.runs
     int64_t n = 0;
     bool loaded = false;
     uint32_t step = 0;          // fused: device sub-step index mirrored on the host
@@ -695,6 +696,29 @@ int choose_config(const mpm_handle *h) {
     return blocks <= 9.0 * sms ? MPM_KERNEL_T256_G2_C2 : MPM_KERNEL_T256_G2;
 }
 
+// Where 128-thread CTAs step an environment whose blocks may take in more runs than
+// shared memory holds (a 27-block neighbourhood of t particles writes at most
+// t / 128 + 27 chunks): the lists in global memory, 8 KB a CTA.
+mpm_status ensure_runs(mpm_handle *h) {
+    if (fused_step_threads(h->kernel_config) >= 256) return MPM_OK;
+    uint32_t most = 0;
+    for (int e = 0; e < h->n_envs; ++e) most = std::max(most, h->env_off[e + 1] - h->env_off[e]);
+    if (most <= (kRunsShared - 27) * 128) return MPM_OK;
+    const size_t count = (size_t)h->fused_grid * kRunsListed;
+    if (h->fb.runs && h->runs_cap >= count) return MPM_OK;
+    uint2 *runs = nullptr;
+    const mpm_status st = dalloc_t(h, &runs, count);
+    if (st == MPM_OK) {
+        h->fb.runs = runs;
+        h->runs_cap = count;
+    } else {
+        cudaGetLastError();
+        h->fb.runs = nullptr;        // a smaller one would not have an entry for every CTA
+        h->runs_cap = 0;
+    }
+    return st;
+}
+
 // Replace the state of every environment: counts[e] particles of environment
 // e, stored env-major in x, v, F, C; volumes[e] its particle volume.
 mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const float *v, const float *F,
@@ -754,6 +778,10 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
         // arrives at and polls the wait between sub-steps (2K patch 104 -> 100 us a call)
         if (config == kConfigT512)
             h->fused_grid = std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
+        // without the lists, 256 threads keep a block's capacity
+        if (ensure_runs(h) != MPM_OK && (st = apply_kernel_config(h, MPM_KERNEL_T256_G2_C2)) != MPM_OK) return st;
+    } else if (is_fused(h)) {
+        ensure_runs(h);
     }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
     if (is_fused(h)) {
@@ -1745,8 +1773,10 @@ mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config) {
     if (st != MPM_OK) return st;
     if (config < 0 || config >= MPM_KERNEL_CONFIGS) return fail(MPM_ERR_ARG, "kernel configuration %d out of range", config);
     st = apply_kernel_config(h, config);
-    if (st == MPM_OK) h->config_set = true;
-    return st;
+    if (st != MPM_OK) return st;
+    h->config_set = true;
+    if (is_fused(h)) ensure_runs(h);      // or, refused, half of a block's capacity with 128 threads
+    return MPM_OK;
 }
 
 mpm_status mpm_get_kernel_config(mpm_handle *h, int32_t *config, int32_t *threads, int32_t *ctas) {

@@ -38,6 +38,9 @@
 // G_{k-1} for reuse), particle buffers and run tables over two, counters over
 // three or four (a slot no CTA reads any more is zeroed meanwhile); the last CTA
 // of a launch advances the sub-step index.
+#include <algorithm>
+#include <climits>
+
 #include "common.cuh"
 #include "launch.h"
 
@@ -45,7 +48,7 @@ namespace gbmpm {
 
 namespace {
 
-constexpr int CMAX = 512;      // run candidates (source chunk x direction) per block
+constexpr int CMAX = kRunsShared;      // run candidates (source chunk x direction) per block in shared memory
 // What a launch belongs to: plain stepping, or a recorded rollout (mpm_tape_record),
 // whose sub-steps keep their records (kRecord) or not (kRollout).
 enum Use { kStep, kRollout, kRecord };
@@ -108,7 +111,7 @@ struct FusedSmem {
     float4 pxi[PD][T], pf0[PD][T], pf1[PD][T];
     float pf2[PD][T];
     uint32_t cand_start[CMAX];     // first slot of each run
-    uint32_t cand_pre[CMAX + 1];   // exclusive prefix of run lengths
+    uint32_t cand_pre[CMAX];       // exclusive prefix of run lengths
     uint32_t lane_first[27], lane_off[27];
     // per pass parity: per direction, each warp's count of it (one byte per
     // warp, so that a lane sums all warps' counts of its direction in one load)
@@ -188,9 +191,20 @@ __device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async
 __device__ __forceinline__ void cp_async_wait_but_two() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
 
 // Slot of logical index j among the block's incoming runs (binary search of
-// the runs' exclusive prefix).
-template <class Smem>
-__device__ __forceinline__ uint32_t source_slot(const Smem &s, uint32_t ncand, uint32_t j) {
+// the runs' exclusive prefix).  This CTA's part of FusedBufs::runs holds them
+// (prefix, first slot) where they are more than CMAX.
+template <bool MORE, class Smem>
+__device__ __forceinline__ uint32_t source_slot(const Smem &s, const FusedBufs &B, uint32_t ncand, uint32_t j) {
+    if (MORE && ncand > CMAX) {
+        const uint2 *runs = B.runs + (size_t)blockIdx.x * kRunsListed;
+        uint32_t lo = 0, hi = ncand - 1u;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1u) >> 1;
+            if (__ldcg(&runs[mid].x) <= j) lo = mid; else hi = mid - 1u;
+        }
+        const uint2 r = __ldcg(&runs[lo]);
+        return r.y + (j - r.x);
+    }
     int lo = 0, hi = (int)ncand - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -200,14 +214,14 @@ __device__ __forceinline__ uint32_t source_slot(const Smem &s, uint32_t ncand, u
 }
 
 // Start copying the particle with logical index j into this thread's slot.
-template <class Smem>
-__device__ __forceinline__ void prefetch_particle(Smem &s, const PState &base, uint32_t in_off, uint32_t ncand,
+template <bool MORE, class Smem>
+__device__ __forceinline__ void prefetch_particle(Smem &s, const FusedBufs &B, uint32_t in_off, uint32_t ncand,
                                                   uint32_t j, int tid, int set) {
-    const uint32_t src = in_off + source_slot(s, ncand, j);
-    cp_async16_cg(&s.pxi[set][tid], &base.xi[src]);
-    cp_async16_cg(&s.pf0[set][tid], &base.f0[src]);
-    cp_async16_cg(&s.pf1[set][tid], &base.f1[src]);
-    cp_async4(&s.pf2[set][tid], &base.f2[src]);
+    const uint32_t src = in_off + source_slot<MORE>(s, B, ncand, j);
+    cp_async16_cg(&s.pxi[set][tid], &B.P[0].xi[src]);
+    cp_async16_cg(&s.pf0[set][tid], &B.P[0].f0[src]);
+    cp_async16_cg(&s.pf1[set][tid], &B.P[0].f1[src]);
+    cp_async4(&s.pf2[set][tid], &B.P[0].f2[src]);
 }
 
 // Start copying global block b's grid region of G_k, its inbox, and its
@@ -246,6 +260,10 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 
 
 // MINB: resident CTAs per SM the configuration is compiled for (the register budget)
+// MORE: a block's runs beyond CMAX are listed in FusedBufs::runs.  CTAs of 128 threads
+// write more, smaller runs; with them a block takes in as many particles as with
+// 256.  (An instantiation of its own, for environments that can need it: the test
+// in every particle's copy made 256 environments of 5K to 40K 1.6% slower.)
 // USE kRecord: also write, for the reverse mode, every block's input particles at
 // their output positions (inside the range [out_base, out_base + total) the
 // block's output was allocated) with their input positions, the list of
@@ -255,7 +273,7 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 // launch's last (WRITE_VC: the one that writes v and C).  target: CTAs of the
 // launch times its sub-steps up to this one.  Returns whether to go on: false
 // after the last sub-step, or when the wait for the other CTAs ran out.
-template <bool WRITE_VC, int T, int GP, int MINB, Use USE, int PD>
+template <bool WRITE_VC, int T, int GP, int MINB, Use USE, int PD, bool MORE>
 __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const DevParams &P, const FusedBufs &B,
                                               const ToolFrame *__restrict__ tools, const StepRecord &rec0, uint32_t k,
                                               uint32_t step, uint32_t target, bool first, bool last) {
@@ -453,7 +471,8 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 }
                 if (lane < 27) { s.lane_first[lane] = first; s.lane_off[lane] = incl - np; }
                 uint32_t ncand = __shfl_sync(0xffffffffu, incl, 26);
-                if (ncand > CMAX) { ncand = CMAX; err |= kErrCapacity; }
+                constexpr uint32_t most = MORE ? kRunsListed : CMAX;
+                if (ncand > most) { ncand = most; err |= kErrCapacity; }
                 __syncwarp();
                 for (uint32_t c0 = 0; c0 < ncand; c0 += 32) {
                     const uint32_t c = c0 + lane;
@@ -468,7 +487,12 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                         const uint32_t y = __shfl_up_sync(0xffffffffu, incl2, o);
                         if (lane >= o) incl2 += y;
                     }
-                    if (c < ncand) { s.cand_start[c] = r.x; s.cand_pre[c] = carry + incl2 - r.y; }
+                    if (MORE && ncand > CMAX) {
+                        if (c < ncand) B.runs[(size_t)blockIdx.x * kRunsListed + c] = make_uint2(carry + incl2 - r.y, r.x);
+                    } else if (c < ncand) {
+                        s.cand_start[c] = r.x;
+                        s.cand_pre[c] = carry + incl2 - r.y;
+                    }
                     carry += __shfl_sync(0xffffffffu, incl2, 31);
                 }
                 nc = ncand;
@@ -476,7 +500,6 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             __syncwarp();
             if (lane == 0) {
                 s.ncand = nc;
-                s.cand_pre[nc] = carry;
                 s.total = carry;
                 s.npass = (carry + T - 1) / T;
                 // issued here, consumed after the barrier below
@@ -511,10 +534,10 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
         }
         // this thread's particle of the first pass, then the next block's inputs;
         // both land while this block computes
-        if (npass > 0 && (uint32_t)tid < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)tid, tid, 0);
+        if (npass > 0 && (uint32_t)tid < total) prefetch_particle<MORE>(s, B, in_off, ncand, (uint32_t)tid, tid, 0);
         cp_async_commit();
         if (PD == 2) {   // and the second pass's
-            if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle(s, B.P[0], in_off, ncand, (uint32_t)(T + tid), tid, 1);
+            if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle<MORE>(s, B, in_off, ncand, (uint32_t)(T + tid), tid, 1);
             cp_async_commit();
         }
         if (s.bids[cb ^ 1] != kNoBlock) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
@@ -660,7 +683,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 nzp = xi.z + P.dt * vz;
                 // every value read from the slot has been consumed: refill it with the
                 // next pass's particle
-                if (pass + PD < npass && jn < total) prefetch_particle(s, B.P[0], in_off, ncand, jn, tid, ps);
+                if (pass + PD < npass && jn < total) prefetch_particle<MORE>(s, B, in_off, ncand, jn, tid, ps);
                 if (!finite3(nxp, nyp, nzp)) {
                     err |= kErrNumeric;
                     nxp = xi.x; nyp = xi.y; nzp = xi.z;
@@ -813,7 +836,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 rec.f1[pos] = a1;
                 rec.f2[pos] = f2;
                 store_vc(rec.vc, pos, vx, vy, vz, Cm);
-                rec.src[pos] = source_slot(s, ncand, j);
+                rec.src[pos] = source_slot<MORE>(s, B, ncand, j);
             }
             if (valid && pos < nparticles) {
                 B.P[0].xi[out_off + pos] = make_float4(nxp, nyp, nzp, idf);
@@ -1000,7 +1023,7 @@ constexpr bool kManySteps = T * MINB <= 640;
 // before.  One launch for all of them spares the launch gap and the ramp of the
 // CTAs between sub-steps; the CTAs then wait for one another, so nsub > 1 needs
 // a cooperative launch.  v and C are written by the last one (if WRITE_VC).
-template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, Use USE = kStep, int PD = 1>
+template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, Use USE = kStep, int PD = 1, bool MORE = false>
 __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B,
                                                         const ToolFrame *__restrict__ tools, uint32_t frames,
                                                         StepRecord rec, uint32_t nsub) {
@@ -1013,10 +1036,10 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     // per stamp, to a counter that was zero.)
     if (*(volatile uint32_t *)&B.ctrl->err & kErrStall) return;
     if constexpr (!kManySteps<T, MINB>) {
-        fused_substep<WRITE_VC, T, GP, MINB, USE, PD>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
+        fused_substep<WRITE_VC, T, GP, MINB, USE, PD, MORE>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
     } else {
         for (uint32_t k = 0;; ++k)
-            if (!fused_substep<WRITE_VC, T, GP, MINB, USE, PD>(s, P, B, tools + (size_t)k * frames, rec, k, step + k,
+            if (!fused_substep<WRITE_VC, T, GP, MINB, USE, PD, MORE>(s, P, B, tools + (size_t)k * frames, rec, k, step + k,
                                                                   (k + 1) * gridDim.x, k == 0, k + 1 == nsub))
                 break;
     }
@@ -1048,6 +1071,14 @@ void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, c
     }
 }
 
+// The kernel of a configuration, as FusedBufs::runs is there or not.
+template <bool WRITE_VC, int T, int GP, int MINB, int PD>
+auto step_kernel(bool more) {
+    if constexpr (T < 256)
+        if (more) return k_fused_step<WRITE_VC, T, GP, MINB, kStep, PD, true>;
+    return k_fused_step<WRITE_VC, T, GP, MINB, kStep, PD>;
+}
+
 // With 128 registers the variant that writes v and C does not spill either, and
 // all sub-steps are one launch; otherwise the last is its own.
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
@@ -1059,21 +1090,24 @@ void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *too
     const int plain = !write_vc ? nsub : kOne ? 0 : nsub - 1;
     const int per = kManySteps<T, MINB> ? plain : 1;
     for (int k = 0; k < plain; k += per)
-        launch_steps(k_fused_step<false, T, GP, MINB, kStep, PD>, T, smem, P, B, tools + k * frames, none, per, grid, st);
+        launch_steps(step_kernel<false, T, GP, MINB, PD>(B.runs != nullptr), T, smem, P, B, tools + k * frames, none, per, grid, st);
     if (plain < nsub)
-        launch_steps(k_fused_step<true, T, GP, MINB, kStep, PD>, T, smem, P, B, tools + plain * frames, none,
+        launch_steps(step_kernel<true, T, GP, MINB, PD>(B.runs != nullptr), T, smem, P, B, tools + plain * frames, none,
                      nsub - plain, grid, st);
 }
 
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
 int variant_occupancy() {
     const int bytes = (int)sizeof(FusedSmem<T, GP, PD>);
-    cudaFuncSetAttribute(k_fused_step<true, T, GP, MINB, kStep, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    cudaFuncSetAttribute(k_fused_step<false, T, GP, MINB, kStep, PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_fused_step<true, T, GP, MINB, kStep, PD>, T, bytes);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_fused_step<false, T, GP, MINB, kStep, PD>, T, bytes);
-    return a < b ? a : b;
+    int least = INT_MAX;
+    for (const bool more : {false, true})
+        for (const auto kernel : {step_kernel<true, T, GP, MINB, PD>(more), step_kernel<false, T, GP, MINB, PD>(more)}) {
+            int ctas = 0;
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, T, bytes);
+            least = std::min(least, ctas);
+        }
+    return least;
 }
 
 }  // namespace

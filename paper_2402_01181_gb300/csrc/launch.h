@@ -120,6 +120,10 @@ void launch_init_tables(const DevParams &P, const SortScratch &s, const FusedBuf
                         cudaStream_t st);
 
 // kernel_fused.cu
+// Runs (source chunk x direction) of a block: as many as shared memory holds, and as
+// many as 128-thread CTAs list in FusedBufs::runs (512 chunks of 256 particles
+// are 1,024 of 128).
+constexpr uint32_t kRunsShared = 512, kRunsListed = 1024;
 struct FusedBufs {
     PState P[2];
     VCState vc;               // v and C of the last sub-step of a call, slot-aligned with P[current]
@@ -133,6 +137,7 @@ struct FusedBufs {
     uint32_t *gstamp;         // per block: last sub-step it was put on a clear list
     Ctrl *ctrl;
     uint32_t *host_err;       // pinned host word that receives Ctrl::err at the end of a launch
+    uint2 *runs;              // per CTA kRunsListed entries for blocks of more than kRunsShared runs, or NULL
     uint32_t max_polls;       // of the wait between two sub-steps of a launch
     uint32_t nblocks;
     // the second buffer of P, chunks, tabs, alist and inbox follows the first in

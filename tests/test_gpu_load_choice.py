@@ -1,0 +1,52 @@
+"""What a load's choice of the kernel configuration must not cost."""
+import numpy as np
+import pytest
+
+import helpers as H
+from oracle import oracle as O
+from paper_2402_01181_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    import __graft_entry__ as ge
+    ge.build()
+    from paper_2402_01181_gb300 import mpm
+    return mpm
+
+
+@pytest.mark.parametrize("config,clustered,status", [
+    (None, 70000, "MPM_OK"), (None, 100000, "MPM_OK"), (2, 100000, "MPM_OK"), (0, 100000, "MPM_OK"),
+    (None, 150000, "MPM_ERR_CAPACITY"), (0, 150000, "MPM_ERR_CAPACITY")])
+def test_a_block_takes_in_512_chunks_of_256_particles(M, config, clustered, status):
+    """A sparse body with a third to most of its particles in 27 neighbouring
+    blocks: 27 x 21 and 27 x 29 chunks of 128 are more than shared memory lists,
+    27 x 22 of 256 are over the documented limit, whoever chose the
+    configuration."""
+    n = 128
+    rng = np.random.default_rng(clustered)
+    total = 220000
+    # base cells [44, 56)^3: blocks 11 to 13 on each axis
+    x = np.concatenate([(44.5 + 12 * rng.random((clustered, 3))) / n,
+                        0.2 + 0.6 * rng.random((total - clustered, 3))]).astype(np.float32)
+    v = (0.1 * (2 * rng.random((total, 3)) - 1)).astype(np.float32)
+    sc = scenes.Scene("cluster", n_grid=n, dt=2e-5, E=10.0, nu=0.3, rho=1e3, x=x, v=v,
+                      particle_volume=(1.0 / n) ** 3 / 3.3)
+    sim = M.sim_from_scene(sc)
+    if config is None:
+        assert sim.kernel_config()["threads"] == 128
+    else:
+        sim.set_kernel_config(config)
+    for _ in range(3):
+        M.mpm_step(sim.h, 1)
+    assert sim.status() == getattr(M, status)
+    if status == "MPM_OK":
+        ids, keys = sim.read_order()
+        out = sim.read()
+        assert np.array_equal(keys, O.block_keys(n, out["x"])[ids]) and np.all(np.diff(keys.astype(np.int64)) >= 0)
+        st = O.State(sc.x, sc.v)
+        H.oracle_steps(sc, st, 0, 3)
+        assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
+    sim.close()
