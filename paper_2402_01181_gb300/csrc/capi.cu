@@ -132,6 +132,12 @@ struct mpm_handle {
     int device = 0, num_sms = 0, fused_grid = 0, elem_grid = 0;
     int kernel_config = 0;          // the fused sub-step's configuration in use
     bool config_set = false;        // by the caller or the autotuner; otherwise by choose_config at each load
+    // a load chose 512 threads by the particles' volume: for as long as they use few
+    // blocks (adapt_config)
+    bool few_blocks = false;
+    uint32_t load_step = 0;         // the load's sub-step index
+    // CTAs by the volume; CTAs of the configurations for more blocks
+    int few_ctas = 0, many_grid = 0, default_grid = 0;
     int n_envs = 1;
     int sub_chunk = 512;        // sub-steps per captured graph / frame upload
     int tstride = 0;            // tool frames per environment in the uploaded table
@@ -417,12 +423,53 @@ mpm_status enqueue_error_copy(mpm_handle *h) {
     return MPM_OK;
 }
 
+// The number of blocks in use that the last finished launch since the load
+// reported, or 0.
+uint32_t blocks_reported(const mpm_handle *h) {
+    const unsigned long long w = *(volatile unsigned long long *)h->fb.host_blocks;
+    return (int32_t)((uint32_t)w - h->load_step) > 0 ? (uint32_t)(w >> 32) : 0u;
+}
+
+// 512 threads as a load chose them pay off while every block has a CTA.  The volume
+// tells the blocks of a body in one piece; particles that lie scattered, or come
+// apart, use many more (2,000 strewn over the 32^3 grid: 380 blocks on 32 CTAs, 1,380
+// us a frame; with 2 CTAs of 256 threads per SM 300).  By what the last launch
+// reported those take over, and give back at half as many; from four blocks per SM on
+// 3 CTAs per SM do, until the next load (8,192 strewn over the 64^3 grid, 2,400
+// blocks: 5,430 us, 2 per SM 1,070, 3 per SM 940; 30,000 over the 128^3 grid,
+// 14,300 blocks: 10,300, 5,750, 4,850).
+constexpr int kConfigMany = MPM_KERNEL_T256_G2_C2;
+void adapt_config(mpm_handle *h) {
+    const uint32_t blocks = h->few_blocks ? blocks_reported(h) : 0u, sms = (uint32_t)h->num_sms;
+    if (blocks == 0) return;
+    if (blocks > 4 * sms) {
+        h->few_blocks = false;
+        h->kernel_config = MPM_KERNEL_T256_G2;
+        h->fused_grid = h->default_grid;
+        return;
+    }
+    const bool many = blocks > (h->kernel_config == kConfigT512 ? sms : sms / 2);
+    h->kernel_config = many ? kConfigMany : kConfigT512;
+    h->fused_grid = many ? h->many_grid : (int)std::min(sms, std::max((uint32_t)h->few_ctas, blocks));
+}
+
 // Issue nsub sub-steps on stream st (used directly and under capture).
 mpm_status issue_substeps(mpm_handle *h, int nsub, bool write_vc_last, cudaStream_t st) {
     const DevParams P = h->P;
     const uint32_t n = (uint32_t)h->n;
     if (is_fused(h)) {
-        launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->fused_grid, h->kernel_config, st);
+        // a load's 512 threads, before any launch has reported the blocks in use: its
+        // kernel takes the call up to one block per SM, otherwise the one behind it does
+        // (3 us for the one that has nothing to do, in the first call after a load)
+        LaunchGate gate;
+        const bool unsure = h->few_blocks && !blocks_reported(h);
+        if (unsure) gate.most_blocks = (uint32_t)h->num_sms;
+        launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->fused_grid, h->kernel_config, st, gate);
+        if (unsure) {
+            gate.most_blocks = LaunchGate::kAny;
+            gate.at = h->step;
+            launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->many_grid, kConfigMany, st, gate);
+        }
         CK(cudaGetLastError());
         return MPM_OK;
     }
@@ -565,7 +612,7 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     h->fb.nblocks = h->nblocks;
     h->elem_grid = h->num_sms * 8;
     const int occ = fused_step_occupancy(h->kernel_config);
-    h->fused_grid = h->num_sms * std::max(occ, 1);
+    h->fused_grid = h->default_grid = h->num_sms * std::max(occ, 1);
 
     mpm_status st;
     const int nbuf = cfg->pipeline == MPM_PIPELINE_FUSED ? 2 : 1;
@@ -616,11 +663,13 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
         e = cudaMallocHost(&h->h_frames[b], sizeof(ToolFrame) * (size_t)h->sub_chunk * n_envs * MPM_MAX_TOOLS);
         if (e != cudaSuccess) return bail(fail(MPM_ERR_ALLOC, "cudaMallocHost: %s", cudaGetErrorString(e)));
     }
-    e = cudaMallocHost(&h->h_err, 2 * sizeof(uint32_t));
+    e = cudaMallocHost(&h->h_err, 4 * sizeof(uint32_t));
     if (e != cudaSuccess) return bail(fail(MPM_ERR_ALLOC, "cudaMallocHost: %s", cudaGetErrorString(e)));
     *h->h_err = 0;
     h->h_total = h->h_err + 1;
     h->fb.host_err = h->h_err;
+    h->fb.host_blocks = reinterpret_cast<unsigned long long *>(h->h_err + 2);
+    *h->fb.host_blocks = 0;
     if ((e = cudaEventCreateWithFlags(&h->ev_err, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[0], cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&h->ev_frames[1], cudaEventDisableTiming)) != cudaSuccess ||
@@ -769,6 +818,8 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     mpm_status st = upload_env_params(h);
     if (st != MPM_OK) return st;
     h->step = k0;
+    h->load_step = k0;
+    h->few_blocks = false;
     h->n = n;
     h->taken = 0;
     if (is_fused(h) && !h->config_set) {
@@ -776,8 +827,13 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
         if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
         // a few CTAs for every block (a body may spread), not one per SM: each more
         // arrives at and polls the wait between sub-steps (2K patch 104 -> 100 us a call)
-        if (config == kConfigT512)
-            h->fused_grid = std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
+        h->few_blocks = config == kConfigT512;
+        if (h->few_blocks) {
+            h->few_ctas = std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
+            h->fused_grid = h->few_ctas;
+            if (h->many_grid == 0) h->many_grid = h->num_sms * std::max(fused_step_occupancy(kConfigMany), 1);
+            CK(cudaGetLastError());
+        }
         // without the lists, 256 threads keep a block's capacity
         if (ensure_runs(h) != MPM_OK && (st = apply_kernel_config(h, MPM_KERNEL_T256_G2_C2)) != MPM_OK) return st;
     } else if (is_fused(h)) {
@@ -919,6 +975,7 @@ mpm_status mpm_step(mpm_handle *h, int32_t n_substeps) {
     if (!h->loaded) return fail(MPM_ERR_STATE, "no particles loaded");
     if ((st = poll_error(h, false)) != MPM_OK) return st;
     if (n_substeps == 0) return MPM_OK;
+    adapt_config(h);
     if (h->n == 0) {
         for (auto &t : h->tools) std::memcpy(t.cur, t.tgt, sizeof t.cur);
         return MPM_OK;
@@ -1775,6 +1832,7 @@ mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config) {
     st = apply_kernel_config(h, config);
     if (st != MPM_OK) return st;
     h->config_set = true;
+    h->few_blocks = false;
     if (is_fused(h)) ensure_runs(h);      // or, refused, half of a block's capacity with 128 threads
     return MPM_OK;
 }

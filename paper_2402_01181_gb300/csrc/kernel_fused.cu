@@ -259,6 +259,11 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
 }
 
 
+// The two configurations between which the host chooses by the blocks in use (512
+// threads, and 256 with 2 CTAs per SM): they report them, and obey a LaunchGate.
+template <int MINB, Use USE>
+constexpr bool kGated = MINB <= 2 && USE == kStep;
+
 // MINB: resident CTAs per SM the configuration is compiled for (the register budget)
 // MORE: a block's runs beyond CMAX are listed in FusedBufs::runs.  CTAs of 128 threads
 // write more, smaller runs; with them a block takes in as many particles as with
@@ -986,6 +991,13 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                 if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
                 ctrl->done = 0;
                 *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
+                if constexpr (kGated<MINB, USE>) {
+                    // the next sub-step's blocks (an append that is not ordered before its
+                    // CTA's arrival may be missing: the host only weighs configurations by them)
+                    const unsigned long long next = *(volatile unsigned long long *)&ctrl->nactive[m3n][0];
+                    *(volatile unsigned long long *)B.host_blocks =
+                        (unsigned long long)((uint32_t)next + (uint32_t)(next >> 32)) << 32 | (step + 1u);
+                }
                 ctrl->step = step + 1;
             }
         }
@@ -1026,7 +1038,7 @@ constexpr bool kManySteps = T * MINB <= 640;
 template <bool WRITE_VC, int T, int GP, int MINB = kMinBlocks<T, GP>, Use USE = kStep, int PD = 1, bool MORE = false>
 __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B,
                                                         const ToolFrame *__restrict__ tools, uint32_t frames,
-                                                        StepRecord rec, uint32_t nsub) {
+                                                        StepRecord rec, uint32_t nsub, LaunchGate gate) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     FusedSmem<T, GP, PD> &s = *reinterpret_cast<FusedSmem<T, GP, PD> *>(smem_raw);
     const uint32_t step = *(volatile uint32_t *)&B.ctrl->step;
@@ -1035,6 +1047,13 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     // load sets them anew.  (That keeps the lists in bounds: a block is appended once
     // per stamp, to a counter that was zero.)
     if (*(volatile uint32_t *)&B.ctrl->err & kErrStall) return;
+    if constexpr (kGated<MINB, USE>) {
+        if (gate.at != LaunchGate::kAny && step != gate.at) return;
+        if (gate.most_blocks != LaunchGate::kAny) {
+            const unsigned long long nhl = *(volatile unsigned long long *)&B.ctrl->nactive[step % 3u][0];
+            if ((uint32_t)nhl + (uint32_t)(nhl >> 32) > gate.most_blocks) return;
+        }
+    }
     if constexpr (!kManySteps<T, MINB>) {
         fused_substep<WRITE_VC, T, GP, MINB, USE, PD, MORE>(s, P, B, tools, rec, 0, step, gridDim.x, true, true);
     } else {
@@ -1049,7 +1068,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
 // where the CTAs cannot all be resident (a context with a part of the SMs).
 template <typename Kernel>
 void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, const FusedBufs &B, const ToolFrame *tools,
-                  const StepRecord &rec, int nsub, int grid, cudaStream_t st) {
+                  const StepRecord &rec, int nsub, int grid, cudaStream_t st, const LaunchGate &gate = {}) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = threads;
@@ -1062,12 +1081,15 @@ void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, c
     cfg.numAttrs = nsub > 1 ? 1 : 0;
     const uint32_t frames = (uint32_t)(P.n_envs * P.tstride);
     // a failure is left for cudaGetLastError
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P, B, tools, frames, rec, (uint32_t)nsub);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P, B, tools, frames, rec, (uint32_t)nsub, gate);
     if (nsub > 1 && (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported)) {
         cudaGetLastError();
         cfg.numAttrs = 0;
-        for (int k = 0; k < nsub; ++k)
-            cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, record_of(rec, k), 1u);
+        for (int k = 0; k < nsub; ++k) {
+            LaunchGate g = gate;       // of the k-th sub-step, if the ones before it ran
+            if (g.at != LaunchGate::kAny) g.at += (uint32_t)k;
+            cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, record_of(rec, k), 1u, g);
+        }
     }
 }
 
@@ -1083,17 +1105,18 @@ auto step_kernel(bool more) {
 // all sub-steps are one launch; otherwise the last is its own.
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
 void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc, int grid,
-                    cudaStream_t st) {
+                    cudaStream_t st, const LaunchGate &gate = {}) {
     constexpr bool kOne = T * MINB <= 512;
     const size_t smem = sizeof(FusedSmem<T, GP, PD>), frames = (size_t)P.n_envs * P.tstride;
     const StepRecord none{};
     const int plain = !write_vc ? nsub : kOne ? 0 : nsub - 1;
     const int per = kManySteps<T, MINB> ? plain : 1;
     for (int k = 0; k < plain; k += per)
-        launch_steps(step_kernel<false, T, GP, MINB, PD>(B.runs != nullptr), T, smem, P, B, tools + k * frames, none, per, grid, st);
+        launch_steps(step_kernel<false, T, GP, MINB, PD>(B.runs != nullptr), T, smem, P, B, tools + k * frames, none, per, grid, st,
+                     gate);
     if (plain < nsub)
         launch_steps(step_kernel<true, T, GP, MINB, PD>(B.runs != nullptr), T, smem, P, B, tools + plain * frames, none,
-                     nsub - plain, grid, st);
+                     nsub - plain, grid, st, gate);
 }
 
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
@@ -1113,13 +1136,13 @@ int variant_occupancy() {
 }  // namespace
 
 void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc,
-                        int grid, int config, cudaStream_t st) {
+                        int grid, int config, cudaStream_t st, const LaunchGate &gate) {
     switch (config) {
     case 1: launch_variant<256, 1>(P, B, tools, nsub, write_vc, grid, st); break;
     case 2: launch_variant<128, 2, kMinBlocks<128, 2>, 2>(P, B, tools, nsub, write_vc, grid, st); break;
     case 3: launch_variant<128, 1>(P, B, tools, nsub, write_vc, grid, st); break;
-    case 4: launch_variant<256, 2, 2, 2>(P, B, tools, nsub, write_vc, grid, st); break;   // 2 CTAs per SM, 128 registers
-    case 5: launch_variant<512, 2>(P, B, tools, nsub, write_vc, grid, st); break;         // 1 CTA per SM, 128 registers
+    case 4: launch_variant<256, 2, 2, 2>(P, B, tools, nsub, write_vc, grid, st, gate); break;   // 2 CTAs per SM, 128 registers
+    case 5: launch_variant<512, 2>(P, B, tools, nsub, write_vc, grid, st, gate); break;         // 1 CTA per SM, 128 registers
     default: launch_variant<256, 2>(P, B, tools, nsub, write_vc, grid, st); break;
     }
 }

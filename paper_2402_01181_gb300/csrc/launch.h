@@ -137,6 +137,7 @@ struct FusedBufs {
     uint32_t *gstamp;         // per block: last sub-step it was put on a clear list
     Ctrl *ctrl;
     uint32_t *host_err;       // pinned host word that receives Ctrl::err at the end of a launch
+    unsigned long long *host_blocks;   // and one for the sub-step index (low) and its number of blocks (high)
     uint2 *runs;              // per CTA kRunsListed entries for blocks of more than kRunsShared runs, or NULL
     uint32_t max_polls;       // of the wait between two sub-steps of a launch
     uint32_t nblocks;
@@ -196,11 +197,18 @@ struct ReverseArgs {
 // 2 = 128, 2; 3 = 128, 1; 4 = 256, 2 with 2 CTAs per SM; 5 = 512, 2 with 1 CTA
 // per SM (chosen by the library only).  Configurations 2 and 4 copy each pass's
 // particles two passes ahead, the others one pass ahead.
+// On what a launch depends, both read on the device: at most that many blocks in
+// use, and the sub-step index it starts from.  A launch does nothing otherwise.  Only
+// for configurations that take all sub-steps of a call in one launch (4 and 5).
+struct LaunchGate {
+    static constexpr uint32_t kAny = 0xffffffffu;
+    uint32_t most_blocks = kAny, at = kAny;
+};
 // nsub sub-steps with the frame tables at tools (n_envs tstride entries each),
 // the last of which also writes v and C if write_vc.  grid: at most the number
 // of CTAs that are resident at once.
 void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc,
-                        int grid, int config, cudaStream_t st);
+                        int grid, int config, cudaStream_t st, const LaunchGate &gate = {});
 int fused_step_occupancy(int config);
 bool fused_many_steps(int config);     // whether a launch takes many sub-steps
 int fused_step_threads(int config);

@@ -50,3 +50,53 @@ def test_a_block_takes_in_512_chunks_of_256_particles(M, config, clustered, stat
         H.oracle_steps(sc, st, 0, 3)
         assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
     sim.close()
+
+
+def _strewn(n, grid, seed=1):
+    return (0.15 + 0.7 * np.random.default_rng(seed).random((n, 3))).astype(np.float32)
+
+
+def _pieces(k, per, grid, ppc):
+    r = np.random.default_rng(k)
+    s = (per / ppc) ** (1 / 3) / grid
+    return np.concatenate([0.15 + 0.65 * r.random(3) + s * r.random((per, 3)) for _ in range(k)]).astype(np.float32)
+
+
+@pytest.mark.parametrize("x,grid,blocks,threads,per_sm", [
+    (_strewn(2000, 32), 32, (153, 608), 256, 2), (_strewn(8192, 64), 64, (609, 9999), 256, 3),
+    (_pieces(40, 200, 64, 8.0), 64, (153, 608), 256, 2), (_pieces(20, 250, 64, 8.0), 64, (49, 152), 512, 1),
+    (scenes.cube8k(1).x, 32, (8, 48), 512, 1)],
+    ids=["strewn2k", "strewn8k", "pieces40", "pieces20", "cube"])
+@pytest.mark.parametrize("queued", [False, True])
+def test_scattered_particles_leave_the_512_threads(M, x, grid, blocks, threads, per_sm, queued):
+    """Chosen by the volume (as in one dense piece), left by the number of blocks
+    in use: in the first call on the device, afterwards by what was reported.
+    8 sub-steps in three calls follow the oracle to the bounds of the parity
+    tests, whichever kernel took them."""
+    rng = np.random.default_rng(len(x))
+    v = (0.2 * (2 * rng.random(x.shape) - 1)).astype(np.float32)
+    sc = scenes.Scene("pieces", n_grid=grid, dt=1e-4, E=1e3, nu=0.3, rho=1e3, x=x, v=v,
+                      particle_volume=(1.0 / grid) ** 3 / 16)
+    used = len(np.unique(O.block_keys(grid, x)))
+    assert blocks[0] <= used <= blocks[1]
+    sms = __import__("torch").cuda.get_device_properties(0).multi_processor_count
+    sim = M.sim_from_scene(sc)
+    assert sim.kernel_config()["threads"] == 512
+    for k in (4, 1, 3):
+        sim.step(k)
+        if not queued:
+            sim.read()
+    out = sim.read()
+    ids, keys = sim.read_order()
+    assert np.array_equal(keys, O.block_keys(grid, out["x"])[ids]) and np.array_equal(np.sort(ids), np.arange(len(x)))
+    sim.step(1)
+    got = sim.kernel_config()
+    assert got["threads"] == threads and (got["ctas"] == per_sm * sms or threads == 512 and used <= got["ctas"])
+    sim.set_kernel_config(2)         # what is set stays
+    sim.step(1)
+    assert sim.kernel_config()["threads"] == 128
+    assert sim.status() == M.MPM_OK
+    sim.close()
+    st = O.State(sc.x, sc.v)
+    H.oracle_steps(sc, st, 0, 8)
+    assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
