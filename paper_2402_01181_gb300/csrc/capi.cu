@@ -729,8 +729,12 @@ static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuratio
 // Measured on 152 SMs, us per sub-step under configurations 0, 2, 3, 4 and 5:
 // - as long as every block can have a CTA of its own, one block's chain counts, so
 //   the largest CTAs that fit (8K cube 21.7, 37, 43, 21.8, 18.1; 50K at 10 per cell
-//   17.8, 22.7, 25.6, 14.2, 12.8; 30K slab 17.1, 17.7, 21.4, 13.8, 17.5; 50K slab at
-//   3 per cell 17.0, 14.9, 18.7, 16.9, 19.5);
+//   17.8, 22.7, 25.6, 14.2, 12.8; 30K slab 17.1, 17.7, 21.4, 13.8, 17.5);
+// - with 2 CTAs per SM that holds to 3 estimated blocks per SM, as long as an SM has up
+//   to 400 particles.  Slabs on 64^3, us per frame of 25 sub-steps under 2, 3 and 4, at
+//   3.2 per cell: 31K 368, 442, 249; 40K 404, 470, 360; 45K 399, 463, 364; 50K (3.2
+//   blocks per SM) 407, 478, 380; at 4 per cell: 56K 404, 476, 393; at 5 per cell: 60K
+//   417, 453, 413; 65K (430 particles per SM) 423, 454, 430; 72K 421, 465, 443;
 // - beyond, sparse blocks waste the fewest threads of the smallest CTAs (200K slab
 //   47, 43, 39, 45, 61; 256 environments 1389, 1200, 1150, 1520, 2340), dense ones
 //   run from 4 to 5 blocks per CTA on with the most warps (500K at 8 per cell 51.4,
@@ -740,7 +744,7 @@ int choose_config(const mpm_handle *h) {
     const bool sparse = (double)h->n < 6.0 * 64.0 * full;
     const double blocks = full * (sparse ? 2.0 : 1.5);
     if (blocks <= sms) return kConfigT512;
-    if (blocks <= 2.0 * sms) return MPM_KERNEL_T256_G2_C2;
+    if (blocks <= 2.0 * sms || (blocks <= 3.0 * sms && (double)h->n <= 400.0 * sms)) return MPM_KERNEL_T256_G2_C2;
     if (sparse) return blocks <= 4.0 * sms ? MPM_KERNEL_T128_G2 : MPM_KERNEL_T128_G1;
     return blocks <= 9.0 * sms ? MPM_KERNEL_T256_G2_C2 : MPM_KERNEL_T256_G2;
 }

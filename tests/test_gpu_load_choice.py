@@ -100,3 +100,17 @@ def test_scattered_particles_leave_the_512_threads(M, x, grid, blocks, threads, 
     st = O.State(sc.x, sc.v)
     H.oracle_steps(sc, st, 0, 8)
     assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n,ppc,threads,per_sm", [
+    (30000, 3.18, 256, 2), (31000, 3.18, 256, 2), (45000, 3.18, 256, 2), (60000, 5.0, 256, 2),
+    (48000, 3.18, 128, 4), (65000, 5.0, 128, 4), (76000, 5.0, 128, 4)])
+def test_sparse_loads_beside_the_rules_edge(M, n, ppc, threads, per_sm):
+    """Just above 2 estimated blocks per SM 128 threads were 48% slower than 2
+    CTAs of 256, and slower than 3 of them."""
+    sms = __import__("torch").cuda.get_device_properties(0).multi_processor_count
+    x = (0.2 + 0.6 * np.random.default_rng(1).random((n, 3))).astype(np.float32)
+    sim = M.Sim(M.make_config(64, 1e-5, 1e4, 0.3, 1e3, max_particles=n))
+    sim.load(x, 1.0 / (ppc * 64 ** 3))
+    assert sim.kernel_config() == {"config": 0, "threads": threads, "ctas": per_sm * sms}
+    sim.close()
