@@ -281,15 +281,17 @@ enum {
  * out of range or not resident on this GPU. */
 mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config);
 
-/* The selected configuration (0 while none is), and the CTA size and the
+/* The selected configuration (0 while none is, and mpm_autotune's best where
+ * it left the choice to the load), and the CTA size and the
  * persistent grid size (CTAs per launch) in use; any output may be NULL. */
 mpm_status mpm_get_kernel_config(mpm_handle *h, int32_t *config, int32_t *threads, int32_t *ctas);
 
 /* Autotuner: time every configuration on the handle's own state (one
  * untimed call of n_substeps sub-steps, then three timed calls, each trial
  * starting from the same snapshot of the particles and tools), select the
- * one with the smallest median call time (none, and best 0, where the load's
- * own choice of 512 threads is faster) and restore the state as it was
+ * one with the smallest median call time (none where the load's own choice of
+ * 512 threads is faster still: the handle keeps that, and best is the fastest
+ * of those that mpm_set_kernel_config takes) and restore the state as it was
  * (particle order inside the library may change; mpm_read_particles returns
  * the same values).  times_ms (MPM_KERNEL_CONFIGS floats: the median call
  * times, -1 for configurations that do not fit) and best may be NULL.  Needs a loaded fused-pipeline handle

@@ -132,6 +132,7 @@ struct mpm_handle {
     int device = 0, num_sms = 0, fused_grid = 0, elem_grid = 0;
     int kernel_config = 0;          // the fused sub-step's configuration in use
     bool config_set = false;        // by the caller or the autotuner; otherwise by choose_config at each load
+    int tuned = 0;                  // mpm_autotune's best where a load's own choice was faster still
     // a load chose 512 threads by the particles' volume: for as long as they use few
     // blocks (adapt_config)
     bool few_blocks = false;
@@ -749,6 +750,13 @@ int choose_config(const mpm_handle *h) {
     return blocks <= 9.0 * sms ? MPM_KERNEL_T256_G2_C2 : MPM_KERNEL_T256_G2;
 }
 
+// CTAs of 512 threads for the loaded particles: a few for every block (a body may
+// spread), not one per SM, as each more arrives at and polls the wait between
+// sub-steps (2K patch 104 -> 100 us a call).
+int few_ctas(const mpm_handle *h) {
+    return std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
+}
+
 // Where 128-thread CTAs step an environment whose blocks may take in more runs than
 // shared memory holds (a 27-block neighbourhood of t particles writes at most
 // t / 128 + 27 chunks): the lists in global memory, 8 KB a CTA.
@@ -829,18 +837,16 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     if (is_fused(h) && !h->config_set) {
         const int config = choose_config(h);
         if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
-        // a few CTAs for every block (a body may spread), not one per SM: each more
-        // arrives at and polls the wait between sub-steps (2K patch 104 -> 100 us a call)
         h->few_blocks = config == kConfigT512;
         if (h->few_blocks) {
-            h->few_ctas = std::min(h->num_sms, std::max(32, (int)std::ceil(6.0 * full_blocks(h))));
-            h->fused_grid = h->few_ctas;
+            h->fused_grid = h->few_ctas = few_ctas(h);
             if (h->many_grid == 0) h->many_grid = h->num_sms * std::max(fused_step_occupancy(kConfigMany), 1);
             CK(cudaGetLastError());
         }
         // without the lists, 256 threads keep a block's capacity
         if (ensure_runs(h) != MPM_OK && (st = apply_kernel_config(h, MPM_KERNEL_T256_G2_C2)) != MPM_OK) return st;
     } else if (is_fused(h)) {
+        if (h->kernel_config == kConfigT512) h->fused_grid = few_ctas(h);     // a trial of the autotuner
         ensure_runs(h);
     }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
@@ -1844,7 +1850,7 @@ mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config) {
 mpm_status mpm_get_kernel_config(mpm_handle *h, int32_t *config, int32_t *threads, int32_t *ctas) {
     mpm_status st = check_handle(h);
     if (st != MPM_OK) return st;
-    if (config) *config = h->config_set ? h->kernel_config : MPM_KERNEL_T256_G2;
+    if (config) *config = h->config_set ? h->kernel_config : h->tuned;
     if (threads) *threads = fused_step_threads(h->kernel_config);
     if (ctas) *ctas = h->fused_grid;
     return MPM_OK;
@@ -1863,7 +1869,7 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
     if (times_ms)
         for (int c = 0; c < MPM_KERNEL_CONFIGS; ++c) times_ms[c] = -1.f;
     if (h->n == 0) {
-        if (best) *best = h->config_set ? h->kernel_config : MPM_KERNEL_T256_G2;
+        if (best) *best = h->config_set ? h->kernel_config : h->tuned;
         return MPM_OK;
     }
     // snapshot of the state, the tools and the counters; every trial starts from it
@@ -1883,15 +1889,17 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
     const int start = h->kernel_config;
     const bool start_set = h->config_set;
     cudaEvent_t a = nullptr, b = nullptr;
-    CK(cudaEventCreate(&a));
-    CK(cudaEventCreate(&b));
+    if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) {
+        if (a) cudaEventDestroy(a);
+        return fail(MPM_ERR_CUDA, "cudaEventCreate failed");
+    }
     h->config_set = true;     // the trials' loads keep the trial's configuration
     auto restore = [&]() -> mpm_status {
         h->tools = tools0;
         return load_impl(h, counts.data(), sx, sv, sF, sC, vols.data(), 1);
     };
-    int pick = start;
-    float best_ms = 3.0e38f;
+    int pick = start, selectable = 0;
+    float best_ms = 3.0e38f, selectable_ms = 3.0e38f;
     // the selectable ones, and the library's own where a load would take it
     const int last = choose_config(h) == kConfigT512 ? kConfigT512 : MPM_KERNEL_CONFIGS - 1;
     for (int c = 0; c <= last && st == MPM_OK; ++c) {
@@ -1916,6 +1924,7 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
         const float ms = reps[kTuneReps / 2];
         if (times_ms && c < MPM_KERNEL_CONFIGS) times_ms[c] = ms;
         if (ms < best_ms) { best_ms = ms; pick = c; }
+        if (c < MPM_KERNEL_CONFIGS && ms < selectable_ms) { selectable_ms = ms; selectable = c; }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
@@ -1926,7 +1935,9 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
     h->taken = taken0;
     if (st != MPM_OK) return st;
     if (st2 != MPM_OK) return st2;
-    if (best) *best = h->config_set ? pick : MPM_KERNEL_T256_G2;
+    // what is reported can be set on another handle: also where a load's own choice won
+    h->tuned = selectable;
+    if (best) *best = selectable;
     return MPM_OK;
 }
 

@@ -114,3 +114,28 @@ def test_sparse_loads_beside_the_rules_edge(M, n, ppc, threads, per_sm):
     sim.load(x, 1.0 / (ppc * 64 ** 3))
     assert sim.kernel_config() == {"config": 0, "threads": threads, "ctas": per_sm * sms}
     sim.close()
+
+
+def _dense33k():
+    x = scenes.jittered_lattice((20, 3, 20), (34, 17, 34), 64, (2, 3, 2), seed=6)
+    return scenes.Scene("dense33k", n_grid=64, dt=5e-5, E=2e4, nu=0.3, rho=1e3, x=x, particle_volume=(1 / 64) ** 3 / 12)
+
+
+@pytest.mark.parametrize("make", [_dense33k, scenes.cube8k, scenes.slab30k], ids=["dense33k", "cube8k", "slab30k"])
+def test_autotune_names_a_configuration_that_can_be_set(M, make):
+    """best is the fastest of the selectable ones, also where the load's 512
+    threads beat them and stay; those keep the CTAs of a load."""
+    sc = make()
+    sim = M.sim_from_scene(sc)
+    loaded = sim.kernel_config()
+    best, times = sim.autotune(10)
+    assert all(t > 0 for t in times) and times[best] == min(times)
+    tuned = sim.kernel_config()
+    assert tuned["config"] == best
+    if tuned["threads"] == 512:
+        assert loaded["threads"] == 512 and tuned["ctas"] == loaded["ctas"]
+    other = M.sim_from_scene(sc)
+    other.set_kernel_config(best)
+    assert other.kernel_config()["config"] == best
+    sim.close()
+    other.close()
