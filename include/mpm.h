@@ -317,7 +317,8 @@ mpm_status mpm_autotune(mpm_handle *h, int32_t n_substeps, float *times_ms, int3
  * pipeline.  On MPM_PIPELINE_FUSED the last segment (the sub-steps after the
  * last checkpoint) is recorded as it runs, so mpm_tape_backward reverses it
  * without recomputing it.  poses: host array.  Device memory for the record is
- * taken from the handle's allocator and kept (and reused) until mpm_destroy. */
+ * taken from the handle's allocator and kept (and reused) until mpm_destroy, or
+ * until a longer rollout's record replaces it. */
 mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *poses,
                            int32_t checkpoint_every);
 
@@ -330,8 +331,10 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
  * grad_material and grad_poses are host arrays.  Each branch of the forward
  * pass (contact, approaching test, friction clamp, closest tool, walls,
  * m > 0) is held at the side taken; distances and sampled fields give no
- * derivative.  Material and tools must be unchanged since the record
- * (MPM_ERR_STATE).  Synchronises. */
+ * derivative.  E, nu and the number of tools must be those of the record
+ * (MPM_ERR_STATE); density and particle volume are taken from the record.  A
+ * rollout whose wait between two sub-steps ran out is refused
+ * (MPM_ERR_TIMEOUT, MPM_ERR_STATE after a load).  Synchronises. */
 mpm_status mpm_tape_backward(mpm_handle *h, const float *x_bar, const float *v_bar, const float *F_bar,
                              const float *C_bar, int on_device, double *grad_material, double *grad_poses,
                              float *x0_bar, float *v0_bar, float *F0_bar, float *C0_bar);

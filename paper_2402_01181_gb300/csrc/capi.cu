@@ -226,6 +226,20 @@ mpm_status dalloc_t(mpm_handle *h, T **out, size_t count) {
     return st;
 }
 
+// Give one buffer back before the handle ends; no work that uses it may be left.
+template <typename T>
+void dfree(mpm_handle *h, T **buf, size_t *cap) {
+    for (size_t i = 0; i < h->allocs.size(); ++i) {
+        if (h->allocs[i].p != *buf) continue;
+        if (h->alloc_fn) h->free_fn(*buf, (void *)h->stream, h->alloc_ctx);
+        else cudaFree(*buf);
+        h->allocs.erase(h->allocs.begin() + (ptrdiff_t)i);
+        break;
+    }
+    *buf = nullptr;
+    *cap = 0;
+}
+
 void release_all(mpm_handle *h) {
     cudaStreamSynchronize(h->stream);
     if (h->rb_stream) {
@@ -1240,19 +1254,51 @@ size_t rs_floats(int64_t n) { return 24 * (size_t)n + 2 * (((size_t)n + 3) & ~si
 size_t rs_words(const mpm_handle *h) { return 3 * (size_t)h->nblocks + 4; }
 
 // Whether the record of a whole rollout of nck segments of ck sub-steps is kept:
-// up to 8 GiB, and a sixteenth of what the device has free, unless the handle has
-// that much from an earlier rollout.  The replays that it spares cost about as much
-// as the forward pass and share the SMs with the reverse sub-steps (30K particles,
-// 100 sub-steps, gradients: 4.95 -> 4.41 ms, a segment recorded in one launch).
+// up to 8 GiB, and a sixteenth of what the device has free beside the handle's present
+// record buffers (which a larger record replaces), unless they have the room.  The
+// replays that it spares cost about as much as the forward pass and share the SMs
+// with the reverse sub-steps (30K particles, 100 sub-steps, gradients: 4.95 -> 4.41 ms,
+// a segment recorded in one launch).
 bool keeps_record(const mpm_handle *h, int64_t n, int ck, int nck) {
     const Tape &tp = h->tape;
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n, steps = (size_t)ck * nck;
     const size_t floats = rs_floats(n) * steps, grids = 2 * nn * steps, words = rs_words(h) * steps;
     if (tp.cap_rs >= floats && tp.cap_rsg >= grids && tp.cap_rsb >= words) return true;
-    const size_t bytes = sizeof(float) * floats + sizeof(float4) * grids + sizeof(uint32_t) * words;
+    auto total = [](size_t f, size_t g, size_t w) { return sizeof(float) * f + sizeof(float4) * g + sizeof(uint32_t) * w; };
+    const size_t bytes = total(floats, grids, words);
     size_t free_b = 0, total_b = 0;
     if (bytes > (size_t)8 << 30 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
-    return bytes <= free_b / 16;
+    return bytes <= (free_b + total(tp.cap_rs, tp.cap_rsg, tp.cap_rsb)) / 16;
+}
+
+// Record buffers for `steps` sub-steps of n particles.  One that is too small is given
+// back first, so that a handle whose rollouts grow holds the last record only; if the
+// device or the caller's allocator refuses one, all are.
+mpm_status reserve_record(mpm_handle *h, int64_t n, size_t steps) {
+    Tape &tp = h->tape;
+    const size_t nn = (size_t)h->P.n * h->P.n * h->P.n;
+    const size_t floats = rs_floats(n) * steps, grids = 2 * nn * steps, words = rs_words(h) * steps;
+    const bool grow_rs = tp.cap_rs < floats, grow_grid = tp.cap_rsg < grids, grow_blk = tp.cap_rsb < words;
+    if (!grow_rs && !grow_grid && !grow_blk) return MPM_OK;
+    CK(cudaStreamSynchronize(h->stream));
+    if (h->rp_stream) CK(cudaStreamSynchronize(h->rp_stream));
+    if (grow_rs) dfree(h, &tp.rs, &tp.cap_rs);
+    if (grow_grid) dfree(h, &tp.rs_grid, &tp.cap_rsg);
+    if (grow_blk) dfree(h, &tp.rs_blk, &tp.cap_rsb);
+    mpm_status st = ensure(h, &tp.rs, &tp.cap_rs, floats);
+    if (st == MPM_OK) st = ensure(h, &tp.rs_grid, &tp.cap_rsg, grids);
+    if (st == MPM_OK) st = ensure(h, &tp.rs_blk, &tp.cap_rsb, words);
+    if (st != MPM_OK) {
+        dfree(h, &tp.rs, &tp.cap_rs);
+        dfree(h, &tp.rs_grid, &tp.cap_rsg);
+        dfree(h, &tp.rs_blk, &tp.cap_rsb);
+        return st;
+    }
+    // recorded sub-steps write the grid (before and after the grid operation) over
+    // their blocks' regions only; the reverse grid operation also reads the rest of the
+    // blocks it lists, where it needs finite values (its adjoint there is zero)
+    if (grow_grid) CK(cudaMemsetAsync(tp.rs_grid, 0, sizeof(float4) * grids, h->stream));
+    return MPM_OK;
 }
 
 // Sub-step j of record buffer buf (segment sg is recorded in buffer sg % nbuf).
@@ -1499,23 +1545,11 @@ mpm_status mpm_tape_record(mpm_handle *h, int32_t n_substeps, const double *pose
         // when there are several: the reverse pass replays a segment into one while
         // it reverses the one in the other
         int nbuf = keeps_record(h, n, ck, nck) ? nck : std::min(nck, 2);
-        auto reserve = [&](size_t steps) -> mpm_status {
-            mpm_status r = ensure(h, &tp.rs, &tp.cap_rs, rs_floats(n) * steps);
-            if (r == MPM_OK && tp.cap_rsg < 2 * nn * steps) {
-                // recorded sub-steps write the grid (before and after the grid operation)
-                // over their blocks' regions only; the reverse grid operation also reads the
-                // rest of the blocks it lists, where it needs finite values (its adjoint
-                // there is zero)
-                if ((r = ensure(h, &tp.rs_grid, &tp.cap_rsg, 2 * nn * steps)) != MPM_OK) return r;
-                CK(cudaMemsetAsync(tp.rs_grid, 0, sizeof(float4) * 2 * nn * steps, h->stream));
-            }
-            return r != MPM_OK ? r : ensure(h, &tp.rs_blk, &tp.cap_rsb, rs_words(h) * steps);
-        };
-        st = reserve((size_t)ck * nbuf);
+        st = reserve_record(h, n, (size_t)ck * nbuf);
         if (st == MPM_ERR_ALLOC && nbuf > 2) {
             cudaGetLastError();
             nbuf = 2;
-            st = reserve((size_t)ck * nbuf);
+            st = reserve_record(h, n, (size_t)ck * nbuf);
         }
         if (st != MPM_OK) return st;
         tp.nbuf = nbuf;

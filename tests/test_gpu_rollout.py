@@ -1,5 +1,6 @@
 """The recorded rollout: its pose gradients against recorded values, and a
 handle that moves on between a record and its backward."""
+import ctypes as ct
 import json
 import os
 
@@ -103,3 +104,53 @@ def test_backward_takes_the_material_of_the_record(M, pipeline, between):
         assert (a[k] - b[k]).abs().max() <= 1e-4 * a[k].abs().max(), k
     assert np.abs(a["poses"]).max() > 0
     assert np.abs(a["poses"] - b["poses"]).max() <= 1e-3 * np.abs(a["poses"]).max()
+
+
+def _recorded_bytes(M, horizons, most=None):
+    """Device bytes a handle holds after rollouts of these lengths, its allocator
+    refusing requests over `most` bytes."""
+    import torch
+    sc = scenes.cube8k()
+    dev = torch.cuda.current_device()
+    live = {}
+
+    def alloc(nbytes, stream, ctx):
+        if most is not None and nbytes > most:
+            return None
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), dev, torch.cuda.current_stream(dev))
+        live[p] = int(nbytes)
+        return p
+
+    def free(ptr, stream, ctx):
+        del live[ptr]                # KeyError: freed twice
+        torch.cuda.caching_allocator_delete(ptr)
+
+    a, f, h = M.mpm_alloc_fn(alloc), M.mpm_free_fn(free), ct.c_void_p()
+    cfg = M.make_config(sc.n_grid, sc.dt, sc.E, sc.nu, sc.rho, max_particles=sc.n)
+    M.check(M.mpm_create(ct.byref(cfg), ct.c_void_p(torch.cuda.current_stream().cuda_stream), a, f, None, ct.byref(h)))
+    x = np.ascontiguousarray(sc.x, dtype=np.float32)
+    grad = np.zeros(2)
+    for k in horizons:
+        M.check(M.mpm_load_particles(h, sc.n, x.ctypes.data_as(ct.c_void_p), None, None, None,
+                                     ct.c_float(sc.particle_volume), 0))
+        M.check(M.mpm_tape_record(h, k, None, 5))
+        M.check(M.mpm_tape_backward(h, None, None, None, None, 1, grad.ctypes.data_as(ct.POINTER(ct.c_double)), None,
+                                    None, None, None, None))
+    held = sum(live.values())
+    M.check(M.mpm_destroy(h))
+    assert not live
+    return held
+
+
+def test_longer_rollouts_replace_the_record(M):
+    """10, 20, 40, then 80 sub-steps hold what 80 alone do, but for the outgrown
+    checkpoints (0.8 MB a segment): 160 MB, not twice that."""
+    once, grown = _recorded_bytes(M, [80]), _recorded_bytes(M, [10, 20, 40, 80])
+    assert once > 120e6 and grown <= once + 20e6, (once, grown)
+
+
+def test_a_record_refused_in_part_is_given_back(M):
+    """Particles of 80 sub-steps (68 MB) granted, their grids (84 MB) refused: the
+    rollout is replayed through two buffers, and nothing else stays."""
+    small, refused = _recorded_bytes(M, [80], 60e6), _recorded_bytes(M, [80], 75e6)
+    assert small < 60e6 and refused == small, (small, refused)
