@@ -645,8 +645,9 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     if ((st = dalloc_t(h, &h->fb.vc.vc1, N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->fb.vc.vc2, N)) != MPM_OK) return bail(st);
     const int ngrid = cfg->pipeline == MPM_PIPELINE_FUSED ? 3 : 1;
-    if ((st = dalloc_t(h, &h->fb.G[0], ngrid * nn)) != MPM_OK) return bail(st);
-    for (int g = 1; g < 3; ++g) h->fb.G[g] = h->fb.G[0] + (g < ngrid ? g * nn : 0);
+    for (int g = 0; g < ngrid; ++g)     // 2.1 GB each at 512^3: not one request for all
+        if ((st = dalloc_t(h, &h->fb.G[g], nn)) != MPM_OK) return bail(st);
+    for (int g = ngrid; g < 3; ++g) h->fb.G[g] = h->fb.G[0];
     if ((st = dalloc_t(h, &h->fb.ctrl, 1)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->staging, 24 * N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->d_frames, (size_t)h->sub_chunk * n_envs * MPM_MAX_TOOLS)) != MPM_OK) return bail(st);
@@ -659,11 +660,11 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
         if ((st = dalloc_t(h, &h->fb.chunks[0], 2 * (size_t)h->chunk_cap)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.tabs[0], 2 * nblk)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.alist[0], 2 * nblk)) != MPM_OK) return bail(st);
-        if ((st = dalloc_t(h, &h->fb.inbox[0], 2 * nblk * kInbox)) != MPM_OK) return bail(st);
+        for (int b = 0; b < 2; ++b)     // larger than a grid
+            if ((st = dalloc_t(h, &h->fb.inbox[b], nblk * kInbox)) != MPM_OK) return bail(st);
         h->fb.chunks[1] = h->fb.chunks[0] + h->chunk_cap;
         h->fb.tabs[1] = h->fb.tabs[0] + nblk;
         h->fb.alist[1] = h->fb.alist[0] + nblk;
-        h->fb.inbox[1] = h->fb.inbox[0] + nblk * kInbox;
         for (int b = 0; b < 3; ++b)
             if ((st = dalloc_t(h, &h->fb.clist[b], h->nblocks)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.astamp, h->nblocks)) != MPM_OK) return bail(st);
@@ -865,7 +866,7 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     }
     const size_t nn = (size_t)h->P.n * h->P.n * h->P.n * h->n_envs;
     if (is_fused(h)) {
-        CK(cudaMemsetAsync(h->fb.G[0], 0, 3 * sizeof(float4) * nn, h->stream));
+        launch_clear_grids(h->fb, nn, h->elem_grid, h->stream);
         CK(cudaMemsetAsync(h->sort.counts, 0, sizeof(uint32_t) * h->nblocks, h->stream));
         launch_block_sort(h->P, dx, (uint32_t)n, h->sort, h->fb.ctrl, h->elem_grid, h->stream);
         const int par = cur_par(h);

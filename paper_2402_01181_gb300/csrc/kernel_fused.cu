@@ -228,7 +228,6 @@ __device__ __forceinline__ void prefetch_particle(Smem &s, const FusedBufs &B, u
 // environment's material and tool frames into buffer buf.
 template <int T, class Smem>
 __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, const uint4 *__restrict__ inbox,
-                                               uint32_t blk_in,
                                                const float4 *__restrict__ Gcur, const DevParams &P,
                                                const ToolFrame *__restrict__ tools, int tid) {
     const int nb = P.nb, n = P.n;
@@ -245,7 +244,7 @@ __device__ __forceinline__ void prefetch_block(Smem &s, int buf, uint32_t b, con
                        ok);
         } else if (q < 216 + kInbox) {
             const int x = q - 216;
-            cp_async16(&s.inbox[buf][x], &inbox[(size_t)(blk_in + b) * kInbox + x], true);
+            cp_async16(&s.inbox[buf][x], &inbox[(size_t)b * kInbox + x], true);
         } else if (q < 216 + kInbox + 2) {
             const int x = q - 216 - kInbox;
             cp_async16(reinterpret_cast<uint4 *>(&s.ep[buf]) + x, reinterpret_cast<const uint4 *>(&P.envp[e]) + x, true);
@@ -357,7 +356,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
         s.own = kNoBlock;
     }
     __syncthreads();
-    if (s.bids[0] != kNoBlock) prefetch_block<T>(s, 0, s.bids[0], B.inbox[0], blk_in, Gcur, P, tools, tid);
+    if (s.bids[0] != kNoBlock) prefetch_block<T>(s, 0, s.bids[0], blk_in ? B.inbox[1] : B.inbox[0], Gcur, P, tools, tid);
     if (tid == 0) { s.m3 = (uint32_t)m3; s.nact = nact; s.nheavy = nheavy; }
     // the P2G arena starts at zero; every flush returns the nodes it read to zero
     if (first)
@@ -545,7 +544,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             if (npass > 1 && (uint32_t)(T + tid) < total) prefetch_particle<MORE>(s, B, in_off, ncand, (uint32_t)(T + tid), tid, 1);
             cp_async_commit();
         }
-        if (s.bids[cb ^ 1] != kNoBlock) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], B.inbox[0], blk_in, Gcur, P, tools, tid);
+        if (s.bids[cb ^ 1] != kNoBlock) prefetch_block<T>(s, cb ^ 1, s.bids[cb ^ 1], blk_in ? B.inbox[1] : B.inbox[0], Gcur, P, tools, tid);
         else cp_async_commit();
         const int ox = 4 * bx - 1, oy = 4 * by - 1, oz = 4 * bz - 1;   // arena origin
 
@@ -824,7 +823,7 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
                     B.chunks[0][chunk_out + chunk_first + pass].run[lane] = make_uint2(pbase + incl - run, run);
                     const int tx = bx + dir_dx(lane), ty = by + dir_dy(lane), tz = bz + dir_dz(lane);
                     if (run > 0u && tx >= 0 && ty >= 0 && tz >= 0 && tx < nb && ty < nb && tz < nb) {
-                        uint4 *dst = B.inbox[0] + (size_t)(blk_out + eb0 + block_id(tx, ty, tz, nb)) * kInbox;
+                        uint4 *dst = (blk_out ? B.inbox[1] : B.inbox[0]) + (size_t)(eb0 + block_id(tx, ty, tz, nb)) * kInbox;
                         if (pass < (uint32_t)kNpMax)
                             dst[lane * kNpMax + pass] = make_uint4(pbase + incl - run, run, step + 1, 0u);
                         else

@@ -243,6 +243,21 @@ __global__ void __launch_bounds__(256) k_init_tables(DevParams P, const uint32_t
     }
 }
 
+// Bound by the writes.  One launch, as three memsets would be two more stream
+// operations in a load.
+__global__ void __launch_bounds__(256) k_clear_grids(float4 *a, float4 *b, float4 *c, size_t nodes) {
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (size_t q = (size_t)blockIdx.x * 256 + threadIdx.x; q < nodes; q += (size_t)gridDim.x * 256) {
+        a[q] = zero;
+        b[q] = zero;
+        c[q] = zero;
+    }
+}
+
+void launch_clear_grids(const FusedBufs &B, size_t nodes, int grid, cudaStream_t st) {
+    k_clear_grids<<<grid, 256, 0, st>>>(B.G[0], B.G[1], B.G[2], nodes);
+}
+
 void launch_init_tables(const DevParams &P, const SortScratch &s, const FusedBufs &B, uint32_t step, int grid,
                         cudaStream_t st) {
     // one block per warp while that is a few waves, as the blocks of a body lie

@@ -116,6 +116,8 @@ struct FusedBufs;
 void launch_place_sorted(const DevParams &P, const float *x, const float *v, const float *F, const float *C,
                          uint32_t n, const SortScratch &s, const PState &S, const VCState &V, int grid,
                          cudaStream_t st);
+// the three grids of `nodes` nodes to zero, in one launch
+void launch_clear_grids(const FusedBufs &B, size_t nodes, int grid, cudaStream_t st);
 void launch_init_tables(const DevParams &P, const SortScratch &s, const FusedBufs &B, uint32_t step, int grid,
                         cudaStream_t st);
 
@@ -141,8 +143,8 @@ struct FusedBufs {
     uint2 *runs;              // per CTA kRunsListed entries for blocks of more than kRunsShared runs, or NULL
     uint32_t max_polls;       // of the wait between two sub-steps of a launch
     uint32_t nblocks;
-    // the second buffer of P, chunks, tabs, alist and inbox follows the first in
-    // one allocation: pstride slots, cstride chunks, nblocks blocks further on
+    // the second buffer of P, chunks, tabs and alist follows the first in one
+    // allocation: pstride slots, cstride chunks, nblocks blocks further on
     uint32_t pstride, cstride;
 };
 // What a recording fused sub-step writes for the reverse mode (all device

@@ -1,4 +1,6 @@
 """What a load's choice of the kernel configuration must not cost."""
+import ctypes as ct
+
 import numpy as np
 import pytest
 
@@ -139,3 +141,38 @@ def test_autotune_names_a_configuration_that_can_be_set(M, make):
     assert other.kernel_config()["config"] == best
     sim.close()
     other.close()
+
+
+def test_grids_and_inboxes_are_requested_one_by_one(M):
+    """An allocator that has no piece larger than one block inbox (27 x 4 + 1
+    entries of 16 bytes a block, more than a grid's 64 nodes) serves the
+    handle, which steps as any other."""
+    import torch
+    n = 128
+    grid, most, asked = 16 * n ** 3, 16 * 109 * (n // 4) ** 3, []
+    dev = torch.cuda.current_device()
+
+    def alloc(nbytes, stream, ctx):
+        asked.append(int(nbytes))
+        return torch.cuda.caching_allocator_alloc(int(nbytes), dev, torch.cuda.current_stream(dev)) \
+            if nbytes <= most else None
+
+    def free(ptr, stream, ctx):
+        torch.cuda.caching_allocator_delete(ptr)
+
+    x = scenes.jittered_lattice((60, 60, 60), (66, 66, 66), n, (2, 2, 2), seed=3)
+    a, f, h = M.mpm_alloc_fn(alloc), M.mpm_free_fn(free), ct.c_void_p()
+    cfg = M.make_config(n, 2e-5, 5e3, 0.3, 1e3, max_particles=len(x))
+    M.check(M.mpm_create(ct.byref(cfg), ct.c_void_p(torch.cuda.current_stream().cuda_stream), a, f, None, ct.byref(h)))
+    assert asked.count(grid) == 3 and asked.count(most) == 2
+    out = np.empty_like(x)
+    for _ in range(2):               # the second load finds grids in use
+        M.check(M.mpm_load_particles(h, len(x), x.ctypes.data_as(ct.c_void_p), None, None, None,
+                                     ct.c_float((1.0 / n) ** 3 / 8), 0))
+        M.check(M.mpm_step(h, 5))
+        M.check(M.mpm_read_particles(h, out.ctypes.data_as(ct.c_void_p), None, None, None, 0))
+    M.check(M.mpm_destroy(h))
+    sc = scenes.Scene("piece", n_grid=n, dt=2e-5, E=5e3, nu=0.3, rho=1e3, x=x, particle_volume=(1.0 / n) ** 3 / 8)
+    st = O.State(sc.x)
+    H.oracle_steps(sc, st, 0, 5)
+    assert np.abs(out - st.x).max() <= 1e-4 * sc.dx
