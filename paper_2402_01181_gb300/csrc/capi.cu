@@ -478,11 +478,13 @@ mpm_status issue_substeps(mpm_handle *h, int nsub, bool write_vc_last, cudaStrea
         // (3 us for the one that has nothing to do, in the first call after a load)
         LaunchGate gate;
         const bool unsure = h->few_blocks && !blocks_reported(h);
-        if (unsure) gate.most_blocks = (uint32_t)h->num_sms;
+        if (unsure) {
+            gate.most_blocks = (uint32_t)h->num_sms;
+            gate.at = h->step;
+        }
         launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->fused_grid, h->kernel_config, st, gate);
         if (unsure) {
             gate.most_blocks = LaunchGate::kAny;
-            gate.at = h->step;
             launch_fused_steps(P, h->fb, h->d_frames, nsub, write_vc_last, h->many_grid, kConfigMany, st, gate);
         }
         CK(cudaGetLastError());
@@ -1000,7 +1002,6 @@ mpm_status mpm_step(mpm_handle *h, int32_t n_substeps) {
     if (!h->loaded) return fail(MPM_ERR_STATE, "no particles loaded");
     if ((st = poll_error(h, false)) != MPM_OK) return st;
     if (n_substeps == 0) return MPM_OK;
-    adapt_config(h);
     if (h->n == 0) {
         for (auto &t : h->tools) std::memcpy(t.cur, t.tgt, sizeof t.cur);
         return MPM_OK;
@@ -1009,6 +1010,7 @@ mpm_status mpm_step(mpm_handle *h, int32_t n_substeps) {
         const int m = std::min(h->sub_chunk, n_substeps - first);
         if ((st = upload_frames(h, first, m, n_substeps)) != MPM_OK) return st;
         const bool last = first + m == n_substeps;
+        adapt_config(h);
         if ((st = run_chunk(h, m, last)) != MPM_OK) return st;
         if (is_fused(h)) h->step += (uint32_t)m;
     }

@@ -1085,8 +1085,11 @@ void launch_steps(Kernel kernel, int threads, size_t smem, const DevParams &P, c
         cudaGetLastError();
         cfg.numAttrs = 0;
         for (int k = 0; k < nsub; ++k) {
-            LaunchGate g = gate;       // of the k-th sub-step, if the ones before it ran
-            if (g.at != LaunchGate::kAny) g.at += (uint32_t)k;
+            LaunchGate g = gate;       // decided for the first sub-step; the others follow it
+            if (k > 0 && g.at != LaunchGate::kAny) {
+                g.at += (uint32_t)k;
+                g.most_blocks = LaunchGate::kAny;
+            }
             cudaLaunchKernelEx(&cfg, kernel, P, B, tools + (size_t)k * frames, frames, record_of(rec, k), 1u, g);
         }
     }

@@ -200,7 +200,7 @@ struct ReverseArgs {
 // per SM (chosen by the library only).  Configurations 2 and 4 copy each pass's
 // particles two passes ahead, the others one pass ahead.
 // On what a launch depends, both read on the device: at most that many blocks in
-// use, and the sub-step index it starts from.  A launch does nothing otherwise.  Only
+// use (with `at`), and the sub-step index it starts from.  A launch does nothing otherwise.  Only
 // for configurations that take all sub-steps of a call in one launch (4 and 5).
 struct LaunchGate {
     static constexpr uint32_t kAny = 0xffffffffu;
