@@ -518,7 +518,8 @@ def run_differentiable(args, rank, device, barrier, max_over_ranks, reps=2):
                 "pipeline": "fused", "forward_record_ms": f, "backward_ms": bk, "fused_forward_ms": pl,
                 "backward_over_fused_forward": bk / pl, "backward_over_recorded_forward": bk / f,
                 "split": {"forward_record_ms": fs, "backward_ms": bks, "backward_over_fused_forward": bks / pl},
-                "note": "min over %d repetitions; the backward includes the segment recomputation" % reps})
+                "note": "min over %d repetitions; the fused record is kept whole up to 8 GiB, otherwise the backward "
+                        "includes the segment recomputation, as on the split pipeline" % reps})
     return res
 
 

@@ -144,7 +144,11 @@ struct mpm_handle {
     int tstride = 0;            // tool frames per environment in the uploaded table
     uint32_t nbe = 0;           // blocks per environment
     uint32_t nblocks = 0, chunk_cap = 0;   // over all environments
-    size_t runs_cap = 0;        // entries of fb.runs
+    // run lists (fb.runs while a load's configuration and particles need them), their
+    // entries, and the configurations whose kernels with them are set up
+    uint2 *runs = nullptr;
+    size_t runs_cap = 0;
+    uint32_t runs_configs = 0;
     int64_t n = 0;
     bool loaded = false;
     uint32_t step = 0;          // fused: device sub-step index mirrored on the host
@@ -778,23 +782,31 @@ int few_ctas(const mpm_handle *h) {
 // shared memory holds (a 27-block neighbourhood of t particles writes at most
 // t / 128 + 27 chunks): the lists in global memory, 8 KB a CTA.
 mpm_status ensure_runs(mpm_handle *h) {
-    if (fused_step_threads(h->kernel_config) >= 256) return MPM_OK;
+    h->fb.runs = nullptr;
+    const int config = h->kernel_config;
+    if (fused_step_threads(config) >= 256) return MPM_OK;
     uint32_t most = 0;
     for (int e = 0; e < h->n_envs; ++e) most = std::max(most, h->env_off[e + 1] - h->env_off[e]);
     if (most <= (kRunsShared - 27) * 128) return MPM_OK;
-    const size_t count = (size_t)h->fused_grid * kRunsListed;
-    if (h->fb.runs && h->runs_cap >= count) return MPM_OK;
-    uint2 *runs = nullptr;
-    const mpm_status st = dalloc_t(h, &runs, count);
-    if (st == MPM_OK) {
-        h->fb.runs = runs;
-        h->runs_cap = count;
-    } else {
-        cudaGetLastError();
-        h->fb.runs = nullptr;        // a smaller one would not have an entry for every CTA
-        h->runs_cap = 0;
+    // its kernels opt into their shared memory, once; the grid is that of the others
+    if (!(h->runs_configs >> config & 1u)) {
+        if (h->num_sms * fused_step_occupancy(config, true) < h->fused_grid)
+            return fail(MPM_ERR_ALLOC, "kernel configuration %d with run lists does not fit", config);
+        h->runs_configs |= 1u << config;
     }
-    return st;
+    const size_t count = (size_t)h->fused_grid * kRunsListed;
+    if (h->runs_cap < count) {
+        uint2 *runs = nullptr;
+        const mpm_status st = dalloc_t(h, &runs, count);
+        if (st != MPM_OK) {
+            cudaGetLastError();
+            return st;
+        }
+        h->runs = runs;
+        h->runs_cap = count;
+    }
+    h->fb.runs = h->runs;
+    return MPM_OK;
 }
 
 // Replace the state of every environment: counts[e] particles of environment

@@ -19,6 +19,10 @@ enum : uint32_t {
     kErrStall = 16u,     // the CTAs of a launch of several sub-steps lost one another
 };
 
+// Ctrl::step after such a loss, until the next load (its own word would be another
+// load in every launch: 25 launches of 1M particles 0.7 us each)
+constexpr uint32_t kStepStalled = 0xffffffffu;
+
 // Per-environment material, in a device table indexed by environment.
 struct EnvParams {
     float mass;       // m_p = rho V_p^0

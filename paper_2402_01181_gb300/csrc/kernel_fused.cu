@@ -38,6 +38,12 @@
 // G_{k-1} for reuse), particle buffers and run tables over two, counters over
 // three or four (a slot no CTA reads any more is zeroed meanwhile); the last CTA
 // of a launch advances the sub-step index.
+//
+// Times in this file's comments are us per frame (25 sub-steps and the readout on the
+// device) of the bodies of perf/cases.py under a moving tool: 2K patch, 8K cube, 30K and
+// 200K slab, 1M and 8M block, one body each, both sides in turn on one GPU.  Other
+// bodies and GPUs shift both sides by up to 15% (8K cube 399 to 467, 30K slab 337 to
+// 376); lightly pressed ones are faster (30K slab 260).
 #include <algorithm>
 #include <climits>
 
@@ -1013,8 +1019,10 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(&ctrl->done) : "memory");
         } while (now < target && ++polls < B.max_polls);
         asm volatile("fence.acq_rel.gpu;" ::: "memory");
-        if (now < target)      // nobody reaches the end of the launch, where the host's copy is written
+        if (now < target) {    // nobody reaches the end of the launch, where step and the host's copy are written
+            *(volatile uint32_t *)&ctrl->step = kStepStalled;
             *(volatile uint32_t *)B.host_err = atomicOr(&ctrl->err, kErrStall) | kErrStall;
+        }
         s.go = now >= target;
     }
     __syncthreads();
@@ -1045,7 +1053,7 @@ __global__ void __launch_bounds__(T, MINB) k_fused_step(DevParams P, FusedBufs B
     // that its CTAs left at different sub-steps: nothing runs on them before the next
     // load sets them anew.  (That keeps the lists in bounds: a block is appended once
     // per stamp, to a counter that was zero.)
-    if (*(volatile uint32_t *)&B.ctrl->err & kErrStall) return;
+    if (step == kStepStalled) return;
     if constexpr (kGated<MINB, USE>) {
         if (gate.at != LaunchGate::kAny && step != gate.at) return;
         if (gate.most_blocks != LaunchGate::kAny) {
@@ -1122,16 +1130,15 @@ void launch_variant(const DevParams &P, const FusedBufs &B, const ToolFrame *too
 }
 
 template <int T, int GP, int MINB = kMinBlocks<T, GP>, int PD = 1>
-int variant_occupancy() {
+int variant_occupancy(bool more) {
     const int bytes = (int)sizeof(FusedSmem<T, GP, PD>);
     int least = INT_MAX;
-    for (const bool more : {false, true})
-        for (const auto kernel : {step_kernel<true, T, GP, MINB, PD>(more), step_kernel<false, T, GP, MINB, PD>(more)}) {
-            int ctas = 0;
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, T, bytes);
-            least = std::min(least, ctas);
-        }
+    for (const auto kernel : {step_kernel<true, T, GP, MINB, PD>(more), step_kernel<false, T, GP, MINB, PD>(more)}) {
+        int ctas = 0;
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, T, bytes);
+        least = std::min(least, ctas);
+    }
     return least;
 }
 
@@ -1179,14 +1186,14 @@ void launch_fused_steps_rollout(const DevParams &P, const FusedBufs &B, const To
 
 // Also opts the kernel into its dynamic shared memory size on the current
 // device; called when a handle is created.
-int fused_step_occupancy(int config) {
+int fused_step_occupancy(int config, bool more) {
     switch (config) {
-    case 1: return variant_occupancy<256, 1>();
-    case 2: return variant_occupancy<128, 2, kMinBlocks<128, 2>, 2>();
-    case 3: return variant_occupancy<128, 1>();
-    case 4: return variant_occupancy<256, 2, 2, 2>();
-    case 5: return variant_occupancy<512, 2>();
-    default: return variant_occupancy<256, 2>();
+    case 1: return variant_occupancy<256, 1>(more);
+    case 2: return variant_occupancy<128, 2, kMinBlocks<128, 2>, 2>(more);
+    case 3: return variant_occupancy<128, 1>(more);
+    case 4: return variant_occupancy<256, 2, 2, 2>(more);
+    case 5: return variant_occupancy<512, 2>(more);
+    default: return variant_occupancy<256, 2>(more);
     }
 }
 

@@ -211,7 +211,7 @@ struct LaunchGate {
 // of CTAs that are resident at once.
 void launch_fused_steps(const DevParams &P, const FusedBufs &B, const ToolFrame *tools, int nsub, bool write_vc,
                         int grid, int config, cudaStream_t st, const LaunchGate &gate = {});
-int fused_step_occupancy(int config);
+int fused_step_occupancy(int config, bool more = false);     // more: of its kernels with FusedBufs::runs
 bool fused_many_steps(int config);     // whether a launch takes many sub-steps
 int fused_step_threads(int config);
 // Sub-steps of a recorded rollout: the CTAs per SM of both kinds (also opts them into
