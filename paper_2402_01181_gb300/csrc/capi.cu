@@ -230,6 +230,21 @@ mpm_status dalloc_t(mpm_handle *h, T **out, size_t count) {
     return st;
 }
 
+// k buffers of `count` elements: one request up to 64 MB (a new handle at 64^3 costs
+// 0.2 ms less), or one each, as a caller's allocator may have no piece for all (the
+// grids take 2.1 GB each at 512^3, the inboxes 3.7).
+template <typename T>
+mpm_status dalloc_each(mpm_handle *h, T **out, int k, size_t count) {
+    mpm_status st = MPM_OK;
+    if (k * count * sizeof(T) <= (size_t)64 << 20) {
+        st = dalloc_t(h, &out[0], k * count);
+        for (int i = 1; i < k; ++i) out[i] = out[0] + i * count;
+        return st;
+    }
+    for (int i = 0; i < k && st == MPM_OK; ++i) st = dalloc_t(h, &out[i], count);
+    return st;
+}
+
 // Give one buffer back before the handle ends; no work that uses it may be left.
 template <typename T>
 void dfree(mpm_handle *h, T **buf, size_t *cap) {
@@ -651,8 +666,7 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
     if ((st = dalloc_t(h, &h->fb.vc.vc1, N)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->fb.vc.vc2, N)) != MPM_OK) return bail(st);
     const int ngrid = cfg->pipeline == MPM_PIPELINE_FUSED ? 3 : 1;
-    for (int g = 0; g < ngrid; ++g)     // 2.1 GB each at 512^3: not one request for all
-        if ((st = dalloc_t(h, &h->fb.G[g], nn)) != MPM_OK) return bail(st);
+    if ((st = dalloc_each(h, h->fb.G, ngrid, nn)) != MPM_OK) return bail(st);
     for (int g = ngrid; g < 3; ++g) h->fb.G[g] = h->fb.G[0];
     if ((st = dalloc_t(h, &h->fb.ctrl, 1)) != MPM_OK) return bail(st);
     if ((st = dalloc_t(h, &h->staging, 24 * N)) != MPM_OK) return bail(st);
@@ -666,8 +680,7 @@ mpm_status mpm_create(const mpm_config *cfg, void *cuda_stream, mpm_alloc_fn all
         if ((st = dalloc_t(h, &h->fb.chunks[0], 2 * (size_t)h->chunk_cap)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.tabs[0], 2 * nblk)) != MPM_OK) return bail(st);
         if ((st = dalloc_t(h, &h->fb.alist[0], 2 * nblk)) != MPM_OK) return bail(st);
-        for (int b = 0; b < 2; ++b)     // larger than a grid
-            if ((st = dalloc_t(h, &h->fb.inbox[b], nblk * kInbox)) != MPM_OK) return bail(st);
+        if ((st = dalloc_each(h, h->fb.inbox, 2, nblk * kInbox)) != MPM_OK) return bail(st);
         h->fb.chunks[1] = h->fb.chunks[0] + h->chunk_cap;
         h->fb.tabs[1] = h->fb.tabs[0] + nblk;
         h->fb.alist[1] = h->fb.alist[0] + nblk;
