@@ -993,16 +993,23 @@ __device__ __forceinline__ bool fused_substep(FusedSmem<T, GP, PD> &s, const Dev
             if (failed) __threadfence();
             if (atomicAdd(&ctrl->done, 1u) == target - 1u) {
                 __threadfence();
-                if (*(volatile uint32_t *)&ctrl->part_alloc[m3] != nparticles) atomicOr(&ctrl->err, kErrCapacity);
+                // one round trip for all three; an append to the next sub-step's list that is
+                // not ordered before its CTA's arrival may be missing from it (the host only
+                // weighs configurations by the blocks)
+                const uint32_t handed_out = *(volatile uint32_t *)&ctrl->part_alloc[m3];
+                uint32_t bits = *(volatile uint32_t *)&ctrl->err;
+                unsigned long long next = 0;
+                if constexpr (kGated<MINB, USE>)
+                    next = *(volatile unsigned long long *)&ctrl->nactive[s.m3 == 2u ? 0u : s.m3 + 1u][0];
+                if (handed_out != nparticles) {
+                    bits |= kErrCapacity;
+                    atomicOr(&ctrl->err, kErrCapacity);
+                }
                 ctrl->done = 0;
-                *(volatile uint32_t *)B.host_err = *(volatile uint32_t *)&ctrl->err;
-                if constexpr (kGated<MINB, USE>) {
-                    // the next sub-step's blocks (an append that is not ordered before its
-                    // CTA's arrival may be missing: the host only weighs configurations by them)
-                    const unsigned long long next = *(volatile unsigned long long *)&ctrl->nactive[m3n][0];
+                *(volatile uint32_t *)B.host_err = bits;
+                if constexpr (kGated<MINB, USE>)
                     *(volatile unsigned long long *)B.host_blocks =
                         (unsigned long long)((uint32_t)next + (uint32_t)(next >> 32)) << 32 | (step + 1u);
-                }
                 ctrl->step = step + 1;
             }
         }
