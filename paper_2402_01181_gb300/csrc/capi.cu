@@ -133,9 +133,11 @@ struct mpm_handle {
     int kernel_config = 0;          // the fused sub-step's configuration in use
     bool config_set = false;        // by the caller or the autotuner; otherwise by choose_config at each load
     int tuned = 0;                  // mpm_autotune's best where a load's own choice was faster still
-    // a load chose 512 threads by the particles' volume: for as long as they use few
-    // blocks (adapt_config)
-    bool few_blocks = false;
+    // a load chose 512 threads by the particles' volume, for as long as they use few
+    // blocks; or it chose those or 2 CTAs of 256 per SM, for as long as they use not many
+    // more than it estimated (adapt_config)
+    bool few_blocks = false, by_volume = false;
+    uint32_t est_blocks = 0;
     uint32_t load_step = 0;         // the load's sub-step index
     // CTAs by the volume; CTAs of the configurations for more blocks
     int few_ctas = 0, many_grid = 0, default_grid = 0;
@@ -471,17 +473,19 @@ uint32_t blocks_reported(const mpm_handle *h) {
 // reported those take over, and give back at half as many; from four blocks per SM on
 // 3 CTAs per SM do, until the next load (8,192 strewn over the 64^3 grid, 2,400
 // blocks: 5,430 us, 2 per SM 1,070, 3 per SM 940; 30,000 over the 128^3 grid,
-// 14,300 blocks: 10,300, 5,750, 4,850).
+// 14,300 blocks: 10,300, 5,750, 4,850).  So they do for a load's 2 CTAs per SM once the
+// blocks are four times its estimate (60,000 over the 128^3 grid: 6,790 against 5,700).
 constexpr int kConfigMany = MPM_KERNEL_T256_G2_C2;
 void adapt_config(mpm_handle *h) {
-    const uint32_t blocks = h->few_blocks ? blocks_reported(h) : 0u, sms = (uint32_t)h->num_sms;
+    const uint32_t blocks = h->by_volume ? blocks_reported(h) : 0u, sms = (uint32_t)h->num_sms;
     if (blocks == 0) return;
-    if (blocks > 4 * sms) {
-        h->few_blocks = false;
+    if (blocks > 4 * std::max(sms, h->est_blocks)) {
+        h->few_blocks = h->by_volume = false;
         h->kernel_config = MPM_KERNEL_T256_G2;
         h->fused_grid = h->default_grid;
         return;
     }
+    if (!h->few_blocks) return;
     const bool many = blocks > (h->kernel_config == kConfigT512 ? sms : sms / 2);
     h->kernel_config = many ? kConfigMany : kConfigT512;
     h->fused_grid = many ? h->many_grid : (int)std::min(sms, std::max((uint32_t)h->few_ctas, blocks));
@@ -756,6 +760,9 @@ double full_blocks(const mpm_handle *h) {
     return full;
 }
 
+bool is_sparse(const mpm_handle *h) { return (double)h->n < 6.0 * 64.0 * full_blocks(h); }
+double estimated_blocks(const mpm_handle *h) { return full_blocks(h) * (is_sparse(h) ? 2.0 : 1.5); }
+
 static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuration follows the selectable ones");
 // The fused sub-step's configuration for the loaded particles, where the caller
 // has set none.  By the number of filled 4x4x4 blocks, estimated as the particles
@@ -775,9 +782,8 @@ static_assert(kConfigT512 == MPM_KERNEL_CONFIGS, "the library's own configuratio
 //   run from 4 to 5 blocks per CTA on with the most warps (500K at 8 per cell 51.4,
 //   59, 61, 50.5, 70; 800K 72.4, 81, 86, 76.3, 106; 1M 94, 105, 109, 100, 138).
 int choose_config(const mpm_handle *h) {
-    const double sms = h->num_sms, full = full_blocks(h);
-    const bool sparse = (double)h->n < 6.0 * 64.0 * full;
-    const double blocks = full * (sparse ? 2.0 : 1.5);
+    const double sms = h->num_sms, blocks = estimated_blocks(h);
+    const bool sparse = is_sparse(h);
     if (blocks <= sms) return kConfigT512;
     if (blocks <= 2.0 * sms || (blocks <= 3.0 * sms && (double)h->n <= 400.0 * sms)) return MPM_KERNEL_T256_G2_C2;
     if (sparse) return blocks <= 4.0 * sms ? MPM_KERNEL_T128_G2 : MPM_KERNEL_T128_G1;
@@ -873,13 +879,15 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
     if (st != MPM_OK) return st;
     h->step = k0;
     h->load_step = k0;
-    h->few_blocks = false;
+    h->few_blocks = h->by_volume = false;
     h->n = n;
     h->taken = 0;
     if (is_fused(h) && !h->config_set) {
         const int config = choose_config(h);
         if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
         h->few_blocks = config == kConfigT512;
+        h->by_volume = h->few_blocks || config == kConfigMany;
+        h->est_blocks = (uint32_t)estimated_blocks(h);
         if (h->few_blocks) {
             h->fused_grid = h->few_ctas = few_ctas(h);
             if (h->many_grid == 0) h->many_grid = h->num_sms * std::max(fused_step_occupancy(kConfigMany), 1);
@@ -1904,7 +1912,7 @@ mpm_status mpm_set_kernel_config(mpm_handle *h, int32_t config) {
     st = apply_kernel_config(h, config);
     if (st != MPM_OK) return st;
     h->config_set = true;
-    h->few_blocks = false;
+    h->few_blocks = h->by_volume = false;
     if (is_fused(h)) ensure_runs(h);      // or, refused, half of a block's capacity with 128 threads
     return MPM_OK;
 }

@@ -104,6 +104,46 @@ def test_scattered_particles_leave_the_512_threads(M, x, grid, blocks, threads, 
     assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
 
 
+@pytest.mark.parametrize("strewn,per_sm", [(True, 3), (False, 2)])
+def test_scattered_particles_leave_two_ctas_per_sm(M, strewn, per_sm):
+    """150,000 particles at a volume of 16 per cell: 220 estimated blocks, and about
+    20,000 in use where they lie strewn over the 128^3 grid."""
+    n, N = 128, 150000
+    rng = np.random.default_rng(3)
+    x = (0.1 + 0.8 * rng.random((N, 3)) if strewn else (40 + 21.1 * rng.random((N, 3))) / n).astype(np.float32)
+    sc = scenes.Scene("strewn", n_grid=n, dt=2e-5, E=100.0, nu=0.3, rho=1e3, x=x, particle_volume=(1.0 / n) ** 3 / 16,
+                      v=(0.2 * (2 * rng.random((N, 3)) - 1)).astype(np.float32))
+    sms = __import__("torch").cuda.get_device_properties(0).multi_processor_count
+    sim = M.sim_from_scene(sc)
+    assert sim.kernel_config() == {"config": 0, "threads": 256, "ctas": 2 * sms}
+    sim.step(2)
+    sim.synchronize()
+    sim.step(2)
+    assert sim.kernel_config() == {"config": 0, "threads": 256, "ctas": per_sm * sms}
+    out = sim.read()
+    sim.close()
+    st = O.State(sc.x, sc.v)
+    H.oracle_steps(sc, st, 0, 4)
+    assert np.abs(out["x"] - st.x).max() <= 1e-4 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-5
+
+
+@pytest.mark.parametrize("x,grid", [(_strewn(2000, 32), 32), (scenes.cube8k(1).x, 32)], ids=["strewn2k", "cube"])
+def test_first_call_of_two_uploads(M, x, grid):
+    """530 sub-steps in the first call after a load: two uploads of tool frames,
+    each decided on the device or by what was reported, follow the oracle to the
+    bounds of 200 sub-steps."""
+    sc = scenes.Scene("two uploads", n_grid=grid, dt=2e-5, E=1e3, nu=0.3, rho=1e3, x=x,
+                      particle_volume=(1.0 / grid) ** 3 / 16)
+    sim = M.sim_from_scene(sc)
+    assert sim.kernel_config()["threads"] == 512
+    sim.step(530)
+    out = sim.read()
+    sim.close()
+    st = O.State(sc.x)
+    H.oracle_steps(sc, st, 0, 530)
+    assert np.abs(out["x"] - st.x).max() <= 1e-3 * sc.dx and np.abs(out["F"] - st.F).max() <= 1e-4
+
+
 @pytest.mark.parametrize("n,ppc,threads,per_sm", [
     (30000, 3.18, 256, 2), (31000, 3.18, 256, 2), (45000, 3.18, 256, 2), (60000, 5.0, 256, 2),
     (48000, 3.18, 128, 4), (65000, 5.0, 128, 4), (76000, 5.0, 128, 4)])
