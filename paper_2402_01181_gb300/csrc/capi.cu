@@ -887,7 +887,7 @@ mpm_status load_impl(mpm_handle *h, const int64_t *counts, const float *x, const
         if (config != h->kernel_config && (st = apply_kernel_config(h, config)) != MPM_OK) return st;
         h->few_blocks = config == kConfigT512;
         h->by_volume = h->few_blocks || config == kConfigMany;
-        h->est_blocks = (uint32_t)estimated_blocks(h);
+        h->est_blocks = (uint32_t)std::min(estimated_blocks(h), 1e9);
         if (h->few_blocks) {
             h->fused_grid = h->few_ctas = few_ctas(h);
             if (h->many_grid == 0) h->many_grid = h->num_sms * std::max(fused_step_occupancy(kConfigMany), 1);
